@@ -1,0 +1,66 @@
+"""Kernel forms chosen by size, alignment or option, at the edges of their tiles.
+
+Each form is compared with the oracle or with the other form that computes
+the same bits: word-wise syndromes (rows that end inside a word, windows that
+wrap) and the vector form of the d-dimensional maps (unaligned buffers, tails).
+"""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_1702_07740_gb300 import qcldpc as q  # noqa: E402
+from test_gpu_parity import U32, dev, gpu_syndrome, odd_code, packed  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device visible")
+    q.load()
+
+
+@pytest.mark.parametrize("Z", [2, 3, 15, 31, 32, 33, 63, 64, 65, 127, 1000])
+def test_syndrome_words_across_rows_and_wraps(Z):
+    d = odd_code(Z) if Z < 64 else synth.rate002_code(Z)
+    code = oracle.Code.from_dict(d)
+    bits = np.random.default_rng(Z).integers(0, 2, (3, code.n)).astype(np.uint8)
+    got = gpu_syndrome(q.create_code_from(d), bits)
+    np.testing.assert_array_equal(got, np.stack([oracle.syndrome(code, b) for b in bits]))
+
+
+@pytest.mark.parametrize("offset", [0, 1, 4])
+@pytest.mark.parametrize("d, n", [(1, 1), (1, 7), (1, 1030), (2, 2), (2, 6), (2, 1030), (4, 4), (4, 1028)])
+def test_maps_of_any_alignment_and_tail(d, n, offset):
+    """Buffers `offset` floats past a 16-byte boundary; the bounds are those of
+    the dimension test (a block product of d terms in FP32). The words after
+    the outputs stay untouched."""
+    rng = np.random.default_rng(10 * n + d)
+    x, y = rng.standard_normal(n).astype(np.float32), rng.standard_normal(n).astype(np.float32)
+    bits = rng.integers(0, 2, n).astype(np.uint8)
+    snr = 0.3
+
+    def buf(a=None):
+        t = torch.full((n + offset + 8,), 7.0, dtype=torch.float32, device="cuda")
+        if a is not None:
+            t[offset:offset + n] = dev(a)
+        return t, t[offset:offset + n]
+
+    (_, xd), (_, yd), (m_all, m), (l_all, llr) = buf(x), buf(y), buf(), buf()
+    q.qcldpc_bob_message(d, yd, dev(packed(bits.reshape(1, -1)).view(np.int32).reshape(-1)), n, m)
+    q.qcldpc_llr(d, xd, m, n, snr, llr)
+    torch.cuda.synchronize()
+    m_gpu = m.cpu().numpy()
+    m_ref = oracle.bob_message(y.astype(np.float64), bits, d=d)
+    yb = np.repeat(np.linalg.norm(y.reshape(-1, d).astype(np.float64), axis=1), d)
+    assert np.all(np.abs(m_gpu - m_ref) <= 16 * U32 * np.sqrt(d) * yb)
+    ref = oracle.llr(x.astype(np.float64), m_gpu.astype(np.float64), snr, d=d)
+    xb = np.repeat(np.linalg.norm(x.reshape(-1, d).astype(np.float64), axis=1), d)
+    mb = np.repeat(np.linalg.norm(m_gpu.reshape(-1, d).astype(np.float64), axis=1), d)
+    assert np.all(np.abs(llr.cpu().numpy() - ref) <= 16 * U32 * (2 * snr / d) * xb * mb + 2 * U32 * np.abs(ref))
+    for t in (m_all, l_all):
+        assert (t[:offset] == 7.0).all() and (t[offset + n:] == 7.0).all()

@@ -232,6 +232,25 @@ def launch_count(group_passes, per_pass: int, unroll: int) -> int:
     return 1 + 2 * len(group_passes) + sum(-(-p // unroll) * unroll * per_pass for p in group_passes)
 
 
+def layered_launches(d, groups: int) -> int:
+    """Kernels of one layered iteration: stop test, control, and per row group
+    its check pass plus, unless its rows have at most four heavy and one
+    degree-1 circulants each and together meet every heavy column at most
+    once, the posterior update."""
+    row, col, mb = np.asarray(d["row"]), np.asarray(d["col"]), d["mb"]
+    heavy = np.bincount(col, minlength=d["nb"])[col] > 1
+    nh = np.bincount(row[heavy], minlength=mb)
+    nd = np.bincount(row[~heavy], minlength=mb)
+    exact = ((nd == 1) & (nh >= 1) & (nh <= 4)) | ((nd == 0) & (nh >= 2) & (nh <= 4))
+    total = 2
+    for g in range(groups):
+        rows = [r for r in range(mb) if r * groups // mb == g]
+        cols = col[heavy & np.isin(row, rows)]
+        fuses = exact[rows].all() and len(np.unique(cols)) == len(cols)
+        total += 1 if fuses else 2
+    return total
+
+
 def groups_of(args, F):
     """Frame groups the decode runs as (the library's rule for frame_groups:
     by default two for flooding, one chain for layered decoding)."""
@@ -483,9 +502,11 @@ def run_ours(args, world, rank, local):
     frames_total = len(used) * F
     fer = frame_err / frames_total
     # per step: llr, and per frame group init + final; per loop pass of a
-    # group's own loop, check pass + control + variable pass (flooding) or
-    # test pass + control + 2 per row group (layered)
-    per_pass = 2 + 2 * (args.layers or d["mb"]) if layered else 3
+    # group's own loop, check pass + posterior pass (flooding; with a separate
+    # variable pass a control step too) or test pass + control + 1 or 2 per row
+    # group (layered)
+    per_pass = (layered_launches(d, args.layers or d["mb"]) if layered
+                else 2 if args.vn_pass == "accumulate" else 3)
     # each group's loop runs flooding iterations four per trip until its own
     # frames have stopped, and the stream launch mode enqueues max_iter + 1
     # passes; passes after every frame stopped exit at once but still launch

@@ -19,20 +19,21 @@
 // diagonal neighbour's constant Phi value and decides that neighbour's bit
 // itself (Step 4 of Algorithm 1 for degree-1 nodes).
 //
-// One iteration t is two streaming kernels plus a one-block control kernel:
-//   cn_tma_kernel per check c (row r, offset i): L_vc = clip(L_v - m_cv(t-1)) for
+// One iteration t is two streaming kernels:
+//   check pass  (cn_tma_kernel) per check c (row r, offset i): L_vc = clip(L_v - m_cv(t-1)) for
 //               heavy neighbours v = (col, (i+s) mod Z), Phi-domain exclusive
 //               sums, m_cv(t) written back in place; decisions of the degree-1
 //               neighbours of iteration t. It also evaluates the stop test of
 //               iteration t-1 (H C(t-1) = s) from the L(t-1) values it reads
 //               anyway, so the test costs no extra pass over memory.
-//   ctrl_kernel freezes frames that passed the test (their L and bits of
-//               iteration t-1 are kept: vn_kernel skips them) and sets the
-//               graph's loop condition.
-//   vn_kernel   per heavy variable v: L_v = Q_v + sum over its ~60 circulants
-//               of m_cv, read at offsets (j - s) mod Z (coalesced, one wrap),
-//               as two interleaved partial sums added in a fixed order.
-// A last pass (t = max_iter + 1) runs cn_tma_kernel as a pure stop test.
+//   post_kernel freezes frames that passed the test (their L and bits of
+//               iteration t-1 are kept), sets the graph's loop condition, and
+//               turns the integer sums that the check pass formed into L_v.
+// With vn_pass = 1 a one-block control kernel (ctrl_kernel) takes the stop
+// decisions, and vn_kernel sums every heavy variable's messages: L_v = Q_v +
+// sum over its ~60 circulants of m_cv, read at offsets (j - s) mod Z
+// (coalesced, one wrap), as two interleaved partial sums added in a fixed order.
+// A last pass (t = max_iter + 1) runs the check pass as a pure stop test.
 // The decode graph's WHILE body holds four flooding iterations (passes of
 // frames that already stopped exit at once). Within it every pass hangs off
 // its predecessor by a programmatic edge: it is scheduled while the
@@ -42,7 +43,8 @@
 // visited in order. An iteration is a stop-test pass (cn_tma_kernel, test
 // only), the control kernel, then per group the group's check pass (messages
 // of iteration t written to the other of two buffers, next to those of t-1)
-// and lvn_kernel, which adds the group's message changes to the posteriors.
+// and lvn_kernel, which adds the group's message changes to the posteriors
+// (cn_group_kernel does both for groups that touch each node at most once).
 //
 // All call arguments travel as one __grid_constant__ parameter (Work), so
 // they sit in the constant bank as warp-uniform operands; instantiated graphs
@@ -311,29 +313,66 @@ __global__ void __launch_bounds__(kThreads) vn_kernel(const __grid_constant__ Ta
     }
 }
 
-// Variable pass of flooding with accumulated posteriors (accum = 1): for
-// every heavy node v = (column hc, j), L_v = Q_v + acc_inv (acc[j] +
-// acc[j + Z]), the exact integer sum of the fixed-point messages the check
-// pass just added, written twice (j and j + Z); both accumulator words are
-// cleared for the next iteration. Frames that stopped keep the posteriors of
-// their last test. Grid (tile of kPostVpt * kThreads nodes, heavy column,
-// frame).
+// What the posterior pass does besides the posteriors.
+enum PostCtl {
+    kPostControl = 1,  // apply the stop tests and count the running frames on
+    kPostClear = 2,    // set the loop condition to "end" (a trip's first pass)
+    kPostKeep = 4,     // ... and to "go on" while a frame runs (its last pass)
+};
+
+// Variable pass and loop control of flooding with accumulated posteriors
+// (accum = 1). For every heavy node v = (column hc, j), L_v = Q_v + acc_inv
+// (acc[j] + acc[j + Z]), the exact integer sum of the fixed-point messages
+// the check pass just added, written twice (j and j + Z); both accumulator
+// words are cleared for the next iteration. Frames that stopped keep the
+// posteriors of their last test. Grid (tile of kPostVpt * kThreads nodes,
+// heavy column, frame).
 // The words are read and cleared with atomic exchanges, which the L2 serves
 // where the reductions landed: on GB300 plain loads of words that many SMs
 // have just reduced into took more than twice as long (18 us against 7.5 us
 // for 16 frames of the n = 10^6 code, measured in isolation).
+// Every block takes its frame's stop decision itself, from words that only
+// the check pass writes (ct, the iteration it ran, and fail, the last
+// iteration whose test failed: tagged with the iteration, so that nothing has
+// to be cleared), and the frame's first block records it. A control kernel
+// of one block between the two passes made every iteration three dependent
+// launches: 50 iterations of one n = 25,600 frame took 554 us that way and
+// 470 us this way, 100 of one n = 10^6 frame 1,572 and 1,462 us.
 constexpr int kPostVpt = 2;
 // PAIR (even Z): a thread takes adjacent nodes j, j + 1 (j even) with one
 // 64-bit exchange per accumulator half, and vector loads and stores.
 template <bool PAIR>
 __global__ void __launch_bounds__(kThreads) post_kernel(const __grid_constant__ Table T,
-                                                        const __grid_constant__ Work W) {
-    pdl_wait();  // the control step's flags (and the check pass's sums) are complete and visible
+                                                        const __grid_constant__ Work W,
+                                                        cudaGraphConditionalHandle handle, int ctl) {
+    pdl_wait();  // the check pass's sums and flags are complete and visible
     pdl_launch_dependents();  // the next iteration's check pass may be scheduled; it waits for this pass
     const int f = blockIdx.z;
-    if (W.active[f] == 0) return;
-    const int Z = T.Z;
     const int hc = blockIdx.y;
+    const bool first = blockIdx.x == 0 && hc == 0 && threadIdx.x == 0;
+    if ((ctl & kPostClear) && first && f == 0) cudaGraphSetConditional(handle, 0u);
+    const int t = W.ct[f];
+    if (t == 0) return;
+    if (ctl & kPostControl) {
+        const bool failed = *W.err != 0;  // a staged copy never completed: stop, flag -1
+        const bool last = t == W.max_iter + 1;
+        const bool passed = (last || (t >= 2 && t - 1 >= W.et_start)) && W.fail[f] != t;
+        const bool stop = failed || passed || last;
+        if (first) {
+            if (stop) {
+                W.conv[f] = failed ? -1 : passed ? 1 : 0;
+                W.iters[f] = t - 1;
+                W.active[f] = 0;
+                if (W.state) W.state[f] = 2;
+            } else {
+                W.t[f] = t + 1;
+                if (ctl & kPostKeep) cudaGraphSetConditional(handle, 1u);
+            }
+        }
+        if (stop) return;
+    }
+    if (hc >= T.n_hcols) return;
+    const int Z = T.Z;
     const float *__restrict__ q = W.llr + (size_t)f * W.n + (size_t)T.hcol_base[hc] * Z;
     float *__restrict__ L = W.L + ((size_t)f * T.n_hcols + hc) * 2 * Z;
     int32_t *__restrict__ a = W.acc + ((size_t)f * T.n_hcols + hc) * 2 * Z;
@@ -380,6 +419,8 @@ dim3 post_grid(const Table &T, int F) {
 template <typename M>
 __global__ void __launch_bounds__(kThreads) lvn_kernel(const __grid_constant__ Table T,
                                                        const __grid_constant__ Work W) {
+    pdl_wait();  // the group's check pass is complete and visible
+    pdl_launch_dependents();  // the next group's check pass may be scheduled; it waits for this pass
     const int f = blockIdx.z;
     if (W.active[f] == 0) return;
     const int t = W.t[f] - 1;
@@ -487,7 +528,7 @@ __global__ void replay_prep_kernel(const __grid_constant__ Work W) {
 // ------------------------------------------------------------ host side
 
 struct Layout {
-    size_t t, err, active, fail, msg, L, acc, phiq, bits, post1, total;
+    size_t t, err, active, ct, fail, msg, L, acc, phiq, bits, post1, total;
 };
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -508,6 +549,7 @@ Layout layout_of(const Table &T, int F, bool soft, int fmt, bool layered = false
     o.t = take(sizeof(int32_t) * Fs);
     o.err = take(sizeof(int32_t));
     o.active = take(sizeof(int32_t) * Fs);
+    o.ct = take(sizeof(int32_t) * Fs);
     o.fail = take(sizeof(int32_t) * Fs);
     o.msg = take(msg_elem_size(fmt) * ((layered ? 2 : 1) * Fs * nh * Z + kSlack));
     o.L = take(sizeof(float) * (Fs * nhc * 2 * Z + kSlack));
@@ -601,6 +643,21 @@ void *lvn_kernel_for(int fmt) {
 void group_rows(const Table &T, int G, int g, int *r0, int *r1) {
     *r0 = (g * T.mb + G - 1) / G;
     *r1 = ((g + 1) * T.mb + G - 1) / G;
+}
+
+// Whether rows [r0, r1) have exact shapes and touch every heavy column at
+// most once: then no two checks of the group share a node, and the group's
+// check pass can update the posteriors itself (cn_group_kernel).
+bool group_fuses(const qcldpc_code *code, int r0, int r1) {
+    const qc::HostTable &h = code->host;
+    std::vector<int32_t> cols;
+    for (int r = r0; r < r1; r++) {
+        const int rp = h.row_ptr[r], nh = h.row_nh[r];
+        if (!exact_shape(nh, h.row_ptr[r + 1] - rp - nh)) return false;
+        for (int k = 0; k < nh; k++) cols.push_back(h.rows[rp + k].col);
+    }
+    std::sort(cols.begin(), cols.end());
+    return std::adjacent_find(cols.begin(), cols.end()) == cols.end();
 }
 
 // psi(y) = log2 coth(y ln2 / 2) in double (base-2 units; psi(inf) = 0).
@@ -767,23 +824,24 @@ cudaError_t raise_priority(cudaGraphNode_t node) {
     return cudaGraphKernelNodeSetAttribute(node, cudaLaunchAttributePriority, &v);
 }
 
-// Loop body of the decode graph. Flooding: check pass -> control ->
-// variable pass. Layered: stop-test pass -> control -> for every row group,
-// its check pass -> its posterior update. The control steps set the loop
-// condition (handle) from the chain's own frames.
-cudaError_t add_loop_body(cudaGraph_t body, const Table &T, const qc::ColsInline &CI,
-                          const Work &w0, cudaGraphConditionalHandle handle) {
+// Loop body of the decode graph. Flooding: check pass -> posterior pass with
+// the control step in it (vn_pass = 1: check pass -> control -> variable pass).
+// Layered: stop-test pass -> control -> for every row group, its check pass ->
+// its posterior update, if the check pass does not do it. The control steps
+// set the loop condition (handle) from the chain's own frames.
+cudaError_t add_loop_body(cudaGraph_t body, const qcldpc_code *code, const Work &w0,
+                          cudaGraphConditionalHandle handle) {
+    const Table &T = code->tab;
     const int F = w0.n_frames;
     Table tcopy = T;
     Work wcopy = w0;
-    qc::ColsInline ccopy = CI;
+    qc::ColsInline ccopy = code->cols_in;
     void *args[] = {&tcopy, &wcopy};
     void *vn_args[] = {&tcopy, &wcopy, &ccopy};
     const CnLaunch cl = cn_launch(T, F, w0.fmt, w0.cn_nt);
     cudaError_t err;
     if (w0.layered) wcopy.pass = kPassTest;
     void *ctrl_args[] = {&wcopy, &handle};
-    const bool pdl = !w0.layered;
     // kLoopUnroll flooding iterations per trip of the WHILE body (each trip
     // costs a body relaunch, ~4 us on GB300): passes of frames that stopped
     // in an earlier iteration of the trip exit at once, and the last control
@@ -796,17 +854,22 @@ cudaError_t add_loop_body(cudaGraph_t body, const Table &T, const qc::ColsInline
         if ((err = add_kernel(&n_cn, body, prev ? &prev : nullptr, prev ? 1 : 0, cl.func, cl.grid, cl.block,
                               args, cl.smem, prev != nullptr && QCLDPC_PDL_LOOP)) != cudaSuccess)
             return err;
+        if (w0.accum) {
+            int ctl = kPostControl | (u == 0 ? kPostClear : 0) | (u == unroll - 1 ? kPostKeep : 0);
+            void *post_args[] = {&tcopy, &wcopy, &handle, &ctl};
+            if ((err = add_kernel(&n_vn, body, &n_cn, 1, post_func(T), post_grid(T, F), dim3(kThreads), post_args,
+                                  0, true)) != cudaSuccess ||
+                (err = raise_priority(n_vn)) != cudaSuccess)
+                return err;
+            prev = n_vn;
+            continue;
+        }
         if ((err = add_kernel(&n_ctrl, body, &n_cn, 1, (void *)ctrl_kernel<true>, dim3(1),
-                              dim3(kCtrlThreads), ctrl_args, 0, pdl)) != cudaSuccess)
+                              dim3(kCtrlThreads), ctrl_args, 0, true)) != cudaSuccess)
             return err;
         if (!w0.layered) {
-            if (w0.accum)
-                err = add_kernel(&n_vn, body, &n_ctrl, 1, post_func(T), post_grid(T, F), dim3(kThreads),
-                                 args, 0, true);
-            else {
-                const VnLaunch vl = vn_launch(T, F, w0.fmt, w0.vn_vpt, w0.vn_split);
-                err = add_kernel(&n_vn, body, &n_ctrl, 1, vl.func, vl.grid, dim3(kThreads), vn_args, 0, true);
-            }
+            const VnLaunch vl = vn_launch(T, F, w0.fmt, w0.vn_vpt, w0.vn_split);
+            err = add_kernel(&n_vn, body, &n_ctrl, 1, vl.func, vl.grid, dim3(kThreads), vn_args, 0, true);
             if (err != cudaSuccess || (err = raise_priority(n_ctrl)) != cudaSuccess ||
                 (err = raise_priority(n_vn)) != cudaSuccess)
                 return err;
@@ -823,10 +886,16 @@ cudaError_t add_loop_body(cudaGraph_t body, const Table &T, const qc::ColsInline
             dim3 grid = cl.grid;
             grid.y = (unsigned)wg.lrows;
             cudaGraphNode_t a, b;
-            if ((err = add_kernel(&a, body, &prev, 1, cl.func, grid, cl.block, gargs,
-                                  cl.smem)) != cudaSuccess ||
-                (err = add_kernel(&b, body, &a, 1, lvn_kernel_for(w0.fmt), vn_grid(T, F),
-                                  dim3(kThreads), gargs)) != cudaSuccess)
+            const bool fuse = group_fuses(code, wg.lrow0, wg.lrow0 + wg.lrows);
+            if ((err = add_kernel(&a, body, &prev, 1, fuse ? cn_tma_kernel_for(T.max_row_deg, w0.fmt, -1) : cl.func,
+                                  grid, cl.block, gargs, cl.smem, true)) != cudaSuccess)
+                return err;
+            if (fuse) {
+                prev = a;
+                continue;
+            }
+            if ((err = add_kernel(&b, body, &a, 1, lvn_kernel_for(w0.fmt), vn_grid(T, F),
+                                  dim3(kThreads), gargs, 0, true)) != cudaSuccess)
                 return err;
             prev = b;
         }
@@ -861,7 +930,7 @@ int build_graph(const qcldpc_code *code, GraphEntry &ge, const Work &w0) {
     if ((err = cudaGraphAddNode(&n_cond, g, &n_init, nullptr, 1, &cp)) != cudaSuccess)
         return qc::cuda_fail(err, "decode: add conditional node");
     cudaGraph_t body = cp.conditional.phGraph_out[0];
-    if ((err = add_loop_body(body, T, code->cols_in, w0, handle)) != cudaSuccess)
+    if ((err = add_loop_body(body, code, w0, handle)) != cudaSuccess)
         return qc::cuda_fail(err, "decode: add loop body");
     if ((err = add_kernel(&n_final, g, &n_cond, 1, (void *)final_kernel, dim3(blocks),
                           dim3(kThreads), args)) != cudaSuccess)
@@ -886,14 +955,24 @@ int stream_decode(qcldpc_code *code, const Work &w, cudaStream_t stream) {
     if (w.layered) wcopy.pass = kPassTest;
     void *args[] = {&tcopy, &wcopy};
     cudaGraphConditionalHandle none = 0;
+    std::vector<char> fuses;
+    for (int g = 0; w.layered && g < w.ngroups; g++) {
+        int r0, r1;
+        group_rows(T, w.ngroups, g, &r0, &r1);
+        fuses.push_back(group_fuses(code, r0, r1));
+    }
     cudaError_t err = cudaGetLastError();
     for (int t = 1; t <= w.max_iter + 1 && err == cudaSuccess; t++) {
         err = cudaLaunchKernel(cl.func, cl.grid, cl.block, args, cl.smem, stream);
         if (err != cudaSuccess) break;
+        if (w.accum) {
+            int ctl = kPostControl;
+            void *post_args[] = {&tcopy, &wcopy, &none, &ctl};
+            err = cudaLaunchKernel(post_func(T), post_grid(T, F), dim3(kThreads), post_args, 0, stream);
+            continue;
+        }
         ctrl_kernel<false><<<1, kCtrlThreads, 0, stream>>>(w, none);
-        if (t <= w.max_iter && !w.layered && w.accum) {
-            err = cudaLaunchKernel(post_func(T), post_grid(T, F), dim3(kThreads), args, 0, stream);
-        } else if (t <= w.max_iter && !w.layered) {
+        if (t <= w.max_iter && !w.layered) {
             qc::ColsInline ccopy = code->cols_in;
             void *vn_args[] = {&tcopy, &wcopy, &ccopy};
             const VnLaunch vl = vn_launch(T, F, w.fmt, w.vn_vpt, w.vn_split);
@@ -907,8 +986,10 @@ int stream_decode(qcldpc_code *code, const Work &w, cudaStream_t stream) {
             void *gargs[] = {&tcopy, &wg};
             dim3 grid = cl.grid;
             grid.y = (unsigned)wg.lrows;
-            err = cudaLaunchKernel(cl.func, grid, cl.block, gargs, cl.smem, stream);
-            if (err == cudaSuccess)
+            const bool fuse = fuses[g];
+            err = cudaLaunchKernel(fuse ? cn_tma_kernel_for(T.max_row_deg, w.fmt, -1) : cl.func, grid, cl.block, gargs,
+                                   cl.smem, stream);
+            if (err == cudaSuccess && !fuse)
                 err = cudaLaunchKernel(lvn_kernel_for(w.fmt), vn_grid(T, F), dim3(kThreads), gargs,
                                        0, stream);
         }
@@ -941,6 +1022,7 @@ Work make_work(const qcldpc_code *code, const qcldpc_params &p, int F, int max_i
     w.post = post;
     w.t = reinterpret_cast<int32_t *>(base + lo.t);
     w.active = reinterpret_cast<int32_t *>(base + lo.active);
+    w.ct = reinterpret_cast<int32_t *>(base + lo.ct);
     w.fail = reinterpret_cast<int32_t *>(base + lo.fail);
     w.err = reinterpret_cast<int32_t *>(base + lo.err);
     w.msg = base + lo.msg;
@@ -1078,6 +1160,7 @@ int decode_impl(const qcldpc_code *code_c, const float *llr, const uint32_t *syn
             works.push_back(make_work(code, p, Fg, max_iter, llr + (size_t)f0 * w.n, syn + (size_t)f0 * w.words_m,
                                       keys + (size_t)f0 * w.words_k, conv + f0, iters + f0, nullptr,
                                       static_cast<char *>(ws) + off, lg));
+            works.back().side = 1;
             off += lg.total;
         }
         return launch_multi(used, works, stream);
@@ -1163,15 +1246,15 @@ extern "C" int qcldpc_decode_soft(const qcldpc_code *code, const float *llr_dev,
 //
 // The graph holds, for every code (or every frame group of one code), the
 // chain a one-code decode runs: initialisation, a device-side loop (a
-// conditional WHILE node) over the flooding passes (check pass, control
-// step, posterior pass, kLoopUnroll times per trip) whose control steps end
-// it once the chain's own frames have stopped, and the output step. The
+// conditional WHILE node) over the flooding passes (check pass and posterior
+// pass, kLoopUnroll times per trip) whose control steps end it once the chain's own frames have stopped, and the output step. The
 // chains are independent branches, so the small grids of short codes fill
 // the GPU together and one chain's short steps run inside another's check
 // pass. Each frame keeps its own iteration counter and stop test, so its
 // result is the one a one-code decode of the same frames gives.
 namespace {
 
+static_assert(kLoopUnroll >= 2, "a trip's first pass clears the loop condition, its last one sets it");
 constexpr int kMultiMaxCodes = QCLDPC_MULTI_MAX_CODES;
 
 struct MultiDecodeGraph {
@@ -1228,8 +1311,7 @@ int build_multi_graph(MultiDecodeGraph &ge, const std::vector<const qcldpc_code 
         cp.conditional.size = 1;
         if ((err = cudaGraphAddNode(&n_cond, g, &n_init, nullptr, 1, &cp)) != cudaSuccess)
             return qc::cuda_fail(err, "decode_multi: add conditional node");
-        if ((err = add_loop_body(cp.conditional.phGraph_out[0], codes[c]->tab, codes[c]->cols_in, works[c],
-                                 handle)) != cudaSuccess)
+        if ((err = add_loop_body(cp.conditional.phGraph_out[0], codes[c], works[c], handle)) != cudaSuccess)
             return qc::cuda_fail(err, "decode_multi: add loop body");
         if ((err = add_kernel(&n_final, g, &n_cond, 1, (void *)final_kernel, dim3(blocks), dim3(kThreads),
                               args)) != cudaSuccess)
@@ -1346,6 +1428,7 @@ extern "C" int qcldpc_decode_multi(int n_codes, const qcldpc_code *const *codes,
         works.push_back(make_work(code, p, F, max_iter, llr_dev[c], syn_dev[c], key_bits_dev[c], converged_dev[c],
                                   iters_dev[c], nullptr, base, lo));
     }
+    for (Work &w : works) w.side = works.size() > 1;
     if (workspace_bytes < off) return fail(QCLDPC_E_NOMEM, "decode_multi: workspace too small");
     if (used.empty()) return QCLDPC_OK;
     return launch_multi(used, works, (cudaStream_t)stream);
@@ -1526,9 +1609,12 @@ extern "C" int qcldpc_time_passes(const qcldpc_code *code_c, int n_frames, void 
     qc::ColsInline ccopy = code->cols_in;
     void *vn_args[] = {&tcopy, &w, &ccopy};
     const VnLaunch vl = vn_launch(T, n_frames, w.fmt, w.vn_vpt, w.vn_split);
+    cudaGraphConditionalHandle none = 0;
+    int ctl = 0;  // the frames neither stop nor count on
+    void *post_args[] = {&tcopy, &w, &none, &ctl};
     for (int r = 0; r < reps && err == cudaSuccess; r++) {
         if (w.accum)
-            err = cudaLaunchKernel(post_func(T), post_grid(T, n_frames), dim3(kThreads), args, 0, stream);
+            err = cudaLaunchKernel(post_func(T), post_grid(T, n_frames), dim3(kThreads), post_args, 0, stream);
         else
             err = cudaLaunchKernel(vl.func, vl.grid, dim3(kThreads), vn_args, 0, stream);
     }
@@ -1731,14 +1817,15 @@ struct qcldpc_pool {
 
 namespace {
 
-// Append n_passes iteration passes of one pool to graph g after node `dep`
-// (nullptr: a root chain). Returns the last node.
-cudaError_t add_pool_passes(cudaGraph_t g, const qcldpc_pool *pool, int n_passes,
+// Append n_passes iteration passes of one pool to graph g as a root chain
+// (side: other pools' chains run beside it). Returns the last node.
+cudaError_t add_pool_passes(cudaGraph_t g, const qcldpc_pool *pool, int n_passes, bool side,
                             cudaGraphNode_t *last) {
     const Table &T = pool->code->tab;
     const int F = pool->n_slots;
     Table tcopy = T;
     Work wcopy = pool->w;
+    wcopy.side = side;
     qc::ColsInline ccopy = pool->code->cols_in;
     void *args[] = {&tcopy, &wcopy};
     void *vn_args[] = {&tcopy, &wcopy, &ccopy};
@@ -1749,10 +1836,12 @@ cudaError_t add_pool_passes(cudaGraph_t g, const qcldpc_pool *pool, int n_passes
     const bool layered = pool->w.layered != 0;
     if (layered) wcopy.pass = kPassTest;
     // layered: one Work per row group (kPassGroup, its base rows)
-    std::vector<Work> wg(layered ? pool->w.ngroups : 0, pool->w);
+    std::vector<Work> wg(layered ? pool->w.ngroups : 0, wcopy);
+    std::vector<char> fuses;
     for (int k = 0; k < (int)wg.size(); k++) {
         wg[k].pass = kPassGroup;
         group_rows(T, pool->w.ngroups, k, &wg[k].lrow0, &wg[k].lrows);
+        fuses.push_back(group_fuses(pool->code, wg[k].lrow0, wg[k].lrows));
         wg[k].lrows -= wg[k].lrow0;
     }
     cudaGraphNode_t prev = nullptr;
@@ -1764,17 +1853,23 @@ cudaError_t add_pool_passes(cudaGraph_t g, const qcldpc_pool *pool, int n_passes
         // posterior update
         cudaGraphNode_t a, b, c;
         err = add_kernel(&a, g, prev ? &prev : nullptr, prev ? 1 : 0, cl.func, cl.grid, cl.block,
-                         args, cl.smem);
+                         args, cl.smem, prev != nullptr && QCLDPC_PDL_LOOP);
+        if (pool->w.accum) {
+            int ctl = kPostControl;
+            void *post_args[] = {&tcopy, &wcopy, &none, &ctl};
+            if (err == cudaSuccess)
+                err = add_kernel(&c, g, &a, 1, post_func(T), post_grid(T, F), dim3(kThreads), post_args, 0, true);
+            // the short step ahead of other pools' pending check blocks
+            if (err == cudaSuccess) err = raise_priority(c);
+            prev = c;
+            continue;
+        }
         if (err == cudaSuccess)
             err = add_kernel(&b, g, &a, 1, (void *)ctrl_kernel<false>, dim3(1), dim3(kCtrlThreads),
-                             ctrl_args);
+                             ctrl_args, 0, true);
         if (!layered) {
-            if (err == cudaSuccess) {
-                if (pool->w.accum)
-                    err = add_kernel(&c, g, &b, 1, post_func(T), post_grid(T, F), dim3(kThreads), args);
-                else
-                    err = add_kernel(&c, g, &b, 1, vl.func, vl.grid, dim3(kThreads), vn_args);
-            }
+            if (err == cudaSuccess)
+                err = add_kernel(&c, g, &b, 1, vl.func, vl.grid, dim3(kThreads), vn_args, 0, true);
             // the short steps ahead of other pools' pending check blocks
             if (err == cudaSuccess) err = raise_priority(b);
             if (err == cudaSuccess) err = raise_priority(c);
@@ -1787,10 +1882,13 @@ cudaError_t add_pool_passes(cudaGraph_t g, const qcldpc_pool *pool, int n_passes
             dim3 grid = cl.grid;
             grid.y = (unsigned)wg[k].lrows;
             cudaGraphNode_t x, y;
-            err = add_kernel(&x, g, &prev, 1, cl.func, grid, cl.block, gargs, cl.smem);
-            if (err == cudaSuccess)
+            const bool fuse = fuses[k];
+            err = add_kernel(&x, g, &prev, 1, fuse ? cn_tma_kernel_for(T.max_row_deg, pool->w.fmt, -1) : cl.func,
+                             grid, cl.block, gargs, cl.smem, true);
+            y = x;
+            if (err == cudaSuccess && !fuse)
                 err = add_kernel(&y, g, &x, 1, lvn_kernel_for(pool->w.fmt), vn_grid(T, F), dim3(kThreads),
-                                 gargs);
+                                 gargs, 0, true);
             prev = y;
         }
     }
@@ -1861,6 +1959,7 @@ extern "C" int qcldpc_pool_create(const qcldpc_code *code_c, int n_slots, int ma
     w.t = reinterpret_cast<int32_t *>(base + lo.base.t);
     w.err = reinterpret_cast<int32_t *>(base + lo.base.err);
     w.active = reinterpret_cast<int32_t *>(base + lo.base.active);
+    w.ct = reinterpret_cast<int32_t *>(base + lo.base.ct);
     w.fail = reinterpret_cast<int32_t *>(base + lo.base.fail);
     w.msg = base + lo.base.msg;
     w.L = reinterpret_cast<float *>(base + lo.base.L);
@@ -1977,7 +2076,7 @@ extern "C" int qcldpc_pools_step(int n_pools, qcldpc_pool *const *pools, int n_p
             hit->graph = nullptr;
             if ((err = cudaGraphCreate(&hit->graph, 0)) != cudaSuccess) return cuda_fail(err, "pools_step: cudaGraphCreate");
             cudaGraphNode_t last;
-            if ((err = add_pool_passes(hit->graph, pool, n_passes, &last)) != cudaSuccess)
+            if ((err = add_pool_passes(hit->graph, pool, n_passes, false, &last)) != cudaSuccess)
                 return cuda_fail(err, "pools_step: add passes");
             if ((err = cudaGraphInstantiate(&hit->exec, hit->graph, cudaGraphInstantiateFlagUseNodePriority)) !=
                 cudaSuccess) {
@@ -2009,7 +2108,7 @@ extern "C" int qcldpc_pools_step(int n_pools, qcldpc_pool *const *pools, int n_p
         err = cudaSuccess;
         for (int i = 0; i < n_pools && err == cudaSuccess; i++) {
             cudaGraphNode_t last;
-            err = add_pool_passes(hit->graph, pools[i], n_passes, &last);
+            err = add_pool_passes(hit->graph, pools[i], n_passes, true, &last);
         }
         if (err == cudaSuccess)
             err = cudaGraphInstantiate(&hit->exec, hit->graph, cudaGraphInstantiateFlagUseNodePriority);
@@ -2060,7 +2159,9 @@ extern "C" int qcldpc_pool_collect(qcldpc_pool *pool, int n, const int32_t *slot
 // the host it is only a stand-in); the device address is fetched once per
 // device with cudaGetSymbolAddress and passed to the kernels.
 constexpr size_t kNoallocScratchBytes = (size_t)16 << 20;  // 16 MiB
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
+// ... and the frames' ct words on top, which the limit on a call does not count.
+constexpr size_t kNoallocCtBytes = (sizeof(int32_t) * 65535 + 255) / 256 * 256;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes + kNoallocCtBytes];
 
 namespace {
 constexpr int kNoallocMaxDevices = 64;
@@ -2078,7 +2179,8 @@ extern "C" int qcldpc_decode_noalloc(const qcldpc_code *code, const float *llr_d
     if (n_frames < 0 || n_frames > 65535)
         return fail(QCLDPC_E_INVAL, "decode_noalloc: n_frames must be in [0, 65535]");
     const size_t need =
-        layout_of(code->tab, n_frames, false, p ? p->msg_format : 0, p && p->schedule == 1).total;
+        layout_of(code->tab, n_frames, false, p ? p->msg_format : 0, p && p->schedule == 1).total -
+        align_up(sizeof(int32_t) * (size_t)n_frames, 256);
     if (need > kNoallocScratchBytes)
         return fail(QCLDPC_E_UNSUPPORTED,
                     "decode_noalloc: this code and frame count need " + std::to_string(need) +
@@ -2106,6 +2208,6 @@ extern "C" int qcldpc_decode_noalloc(const qcldpc_code *code, const float *llr_d
     q.launch_mode = 1;  // plain launches: no graph objects to instantiate
     q.soft_output = 0;
     return decode_impl(code, llr_dev, syn_dev, n_frames, max_iter, &q, key_bits_dev,
-                       converged_dev, iters_dev, nullptr, scratch, kNoallocScratchBytes,
+                       converged_dev, iters_dev, nullptr, scratch, kNoallocScratchBytes + kNoallocCtBytes,
                        (cudaStream_t)stream);
 }

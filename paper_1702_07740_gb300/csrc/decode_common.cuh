@@ -133,7 +133,8 @@ struct Work {
     int32_t *t;            // [F] iteration each frame is at
     int32_t *state;        // [F] slot state for pools (0 free, 1 running, 2 stopped) or null
     int32_t *active;       // [F]
-    int32_t *fail;         // [F] stop-test failures of the current pass
+    int32_t *ct;           // [F] iteration the current flooding check pass runs, 0: frame not running
+    int32_t *fail;         // [F] iteration of the last pass whose stop test failed (0: none yet)
     int32_t *err;          // device error word (a bounded wait gave up)
     void *msg;             // [F][n_h][Z] messages in the storage format fmt (layered:
                            // two such buffers msg_buf elements apart, by iteration parity)
@@ -166,6 +167,7 @@ struct Work {
     int32_t *acc;          // [F][n_hcols][2Z]
     float acc_scale;       // FP32 / FP16 messages: fixed-point scale 2^k (int8: unused)
     float acc_inv;         // 2^-k, or the int8 quantum (the sum then counts quanta)
+    int32_t side;          // 1: other chains run beside this one (see cn_tma_kernel)
     int32_t accum;         // 1: accumulated posteriors; 0: separate summing variable pass
     // Bounded waits of the staged check pass: polls before giving up, and a
     // test switch (QCLDPC_TEST_STALL=1 in the environment) under which each
@@ -334,6 +336,15 @@ struct Codec<int8_t> {
     }
 };
 
+// Stored message `now` less stored message `old`, as lvn_kernel subtracts them.
+__device__ __forceinline__ float msg_change(float now, float old, const Work &) { return now - old; }
+__device__ __forceinline__ float msg_change(__half now, __half old, const Work &) {
+    return __half2float(now) - __half2float(old);
+}
+__device__ __forceinline__ float msg_change(int8_t now, int8_t old, const Work &W) {
+    return __fmaf_rn((float)now, W.qstep, -__fmul_rn((float)old, W.qstep));
+}
+
 // The integer a stored message adds to its node's accumulator: the stored
 // value in units of acc_inv (the int8 code itself; FP32 and FP16 values
 // rounded to the fixed-point grid 2^-k).
@@ -348,12 +359,41 @@ __device__ __forceinline__ void red_add(int32_t *p, int v) {
     asm volatile("red.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Predicated store / reduction: no branch around it (a branch per store and
+// reduction costs three instructions each, and splits the schedule).
+__device__ __forceinline__ void red_add_if(int32_t *p, int v, bool on) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q red.global.add.s32 [%0], %1;\n\t}" ::"l"(p),
+                 "r"(v), "r"((int)on)
+                 : "memory");
+}
+__device__ __forceinline__ void st_if(float *p, float v, bool on) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.global.f32 [%0], %1;\n\t}" ::"l"(p), "f"(v),
+                 "r"((int)on)
+                 : "memory");
+}
+__device__ __forceinline__ void st_if(uint32_t *p, uint32_t v, bool on) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.global.u32 [%0], %1;\n\t}" ::"l"(p), "r"(v),
+                 "r"((int)on)
+                 : "memory");
+}
+__device__ __forceinline__ void st_if(__half *p, __half v, bool on) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.global.u16 [%0], %1;\n\t}" ::"l"(p),
+                 "h"(__half_as_ushort(v)), "r"((int)on)
+                 : "memory");
+}
+__device__ __forceinline__ void st_if(int8_t *p, int8_t v, bool on) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.global.u8 [%0], %1;\n\t}" ::"l"(p), "r"((int)v),
+                 "r"((int)on)
+                 : "memory");
+}
+
 }  // namespace
 
 namespace qc {
 // Check-pass kernels of one storage format (FP32, FP16, int8) for codes whose
 // rows have at most maxdeg circulants: the full-block kernel when nt ==
-// kCnThreads, else the one that takes its width from the launch.
+// kCnThreads, the one that updates a row group's posteriors too when nt < 0,
+// else the one that takes its width from the launch.
 void *cn_kernel_f32(int maxdeg, int nt);
 void *cn_kernel_f16(int maxdeg, int nt);
 void *cn_kernel_i8(int maxdeg, int nt);

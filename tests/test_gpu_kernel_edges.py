@@ -2,19 +2,22 @@
 
 Each form is compared with the oracle or with the other form that computes
 the same bits: word-wise syndromes (rows that end inside a word, windows that
-wrap) and the vector form of the d-dimensional maps (unaligned buffers, tails).
+wrap), the vector form of the d-dimensional maps (unaligned buffers, tails),
+and row groups whose check pass updates the posteriors itself.
 """
 import numpy as np
 import pytest
 
 import oracle
 import synth
+from frames import make_frames
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 from paper_1702_07740_gb300 import qcldpc as q  # noqa: E402
-from test_gpu_parity import U32, dev, gpu_syndrome, odd_code, packed  # noqa: E402
+from test_gpu_parity import (U32, assert_posteriors_close, decode_soft, dev, gpu_syndrome,  # noqa: E402
+                             odd_code, packed)
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -64,3 +67,22 @@ def test_maps_of_any_alignment_and_tail(d, n, offset):
     assert np.all(np.abs(llr.cpu().numpy() - ref) <= 16 * U32 * (2 * snr / d) * xb * mb + 2 * U32 * np.abs(ref))
     for t in (m_all, l_all):
         assert (t[:offset] == 7.0).all() and (t[offset + n:] == 7.0).all()
+
+
+@pytest.mark.parametrize("maker, Z, groups", [
+    (synth.rate002_code, 31, 0), (synth.rate002_code, 33, 0), (synth.rate002_code, 1025, 0), (odd_code, 5, 0),
+    (odd_code, 37, 0), (synth.met_code, 41, 0),
+])
+def test_one_row_groups_match_the_oracle(maker, Z, groups):
+    """Rows that meet each heavy column at most once update the posteriors in
+    their check pass, the others in a pass of their own; both kinds occur."""
+    fr = make_frames(maker(Z), 0.1, 2, d=2)
+    code = q.create_code_from(fr.code_dict)
+    iters = 6
+    layer = oracle.row_layers(fr.code, fr.code.mb)
+    _, conv, its, post = decode_soft(code, dev(fr.q64.astype(np.float32).reshape(-1)), fr.syn, fr.F, iters, et_start=iters + 1,
+                                     schedule=1, layers=groups)
+    for f in range(fr.F):
+        ref, _, it, cv = oracle.decode_layered(fr.code, fr.q64[f], fr.syn[f], iters, layer, et_start=iters + 1)
+        assert_posteriors_close(post[f], ref, f"Z {Z} frame {f}")
+        assert its[f] == it and conv[f] == int(cv)

@@ -31,12 +31,13 @@ __device__ __forceinline__ bool cn_row_generic(const Table &T, const Work &W, in
     const int rp = T.row_ptr[r];
     const int deg = T.row_ptr[r + 1] - rp;
     const int nh = T.row_nh[r];
-    const M *msg_rd = static_cast<const M *>(W.msg) + ((t - 1) & 1) * W.msg_buf + (size_t)f * T.n_h * Z;
-    M *msg = static_cast<M *>(W.msg) + (t & 1) * W.msg_buf + (size_t)f * T.n_h * Z;
-    const float *L = W.L + (size_t)f * T.n_hcols * 2 * Z;
-    int32_t *acc = W.acc + (size_t)f * T.n_hcols * 2 * Z;
-    const float *phiq = W.phiq + (size_t)f * T.n_d1 * Z;
-    const size_t bstride = (size_t)T.n_d1 * ZW;
+    const bool folded = syn_folded(deg - nh);
+    const M *msg_rd = static_cast<const M *>(W.msg) + ((t - 1) & 1) * W.msg_buf + (size_t)f * W.msg_f;
+    M *msg = static_cast<M *>(W.msg) + (t & 1) * W.msg_buf + (size_t)f * W.msg_f;
+    const float *L = W.L + (size_t)f * W.col_f;
+    int32_t *acc = W.acc + (size_t)f * W.col_f;
+    const float *phiq = W.phiq + (size_t)f * W.d1_f;
+    const size_t bstride = W.bit_f;
     uint32_t *bcur = W.bits + ((size_t)(t & 1) * W.n_frames + f) * bstride;
     const uint32_t *bprev = W.bits + ((size_t)((t - 1) & 1) * W.n_frames + f) * bstride;
     const uint32_t *syn = W.syn + (size_t)f * W.words_m;
@@ -45,7 +46,8 @@ __device__ __forceinline__ bool cn_row_generic(const Table &T, const Work &W, in
         const int i = i0 + u * stride;
         const bool valid = i < Z;
         const int cidx = r * Z + i;
-        const uint32_t sbit = __ldg(syn + min(cidx >> 5, (int)W.words_m - 1)) << (31 - (cidx & 31));
+        const uint32_t syn_bit = __ldg(syn + min(cidx >> 5, (int)W.words_m - 1)) << (31 - (cidx & 31));
+        const uint32_t sbit = folded ? 0u : syn_bit;
         float phi[MAXD];
         uint32_t sg[MAXD];
         uint32_t stot = sbit, par = sbit;
@@ -103,7 +105,7 @@ __device__ __forceinline__ bool cn_row_generic(const Table &T, const Work &W, in
                     const float mag = fminf(psi_f(ex), W.clip);
                     float *post1 = W.post1 + ((size_t)(t & 1) * W.n_frames + f) * T.n_d1 * Z;
                     post1[oa + i] = W.llr[(size_t)f * W.n + (size_t)e.col * Z + vo] +
-                                    kLn2 * __uint_as_float(fbits(mag) ^ sk);
+                                    kLn2 * __uint_as_float(fbits(mag) ^ sk ^ (folded ? syn_bit & kSign : 0u));
                 }
             }
         }
@@ -200,15 +202,17 @@ __device__ __forceinline__ bool stage_wait(uint64_t *bar, const Work &W) {
 }
 
 // Soft output of a degree-1 neighbour (row entry e, check i) at iteration t:
-// its posterior Q_p + m_cp in natural units, where the message has sign sk
-// and psi-domain magnitude psi(ex) (clipped).
-__device__ __noinline__ void soft_deg1(const Table &T, const Work &W, int f, int t, int e, int i,
+// its posterior Q_p + m_cp in natural units, where the message has sign sk,
+// less the check's syndrome bit (see syn_folded), and psi-domain magnitude
+// psi(ex) (clipped).
+__device__ __noinline__ void soft_deg1(const Table &T, const Work &W, int f, int r, int t, int e, int i,
                                        float ex, uint32_t sk) {
     const int Z = T.Z;
     const qc::RowEnt re = T.rows[e];
     int vo = i + re.shift;
     if (vo >= Z) vo -= Z;
     const float mag = fminf(psi_f(ex), W.clip);
+    sk ^= syn_sign(W, f, r * Z + i);
     float *post1 = W.post1 + ((size_t)(t & 1) * W.n_frames + f) * T.n_d1 * Z;
     post1[T.row_off_a[e] + i] =
         W.llr[(size_t)f * W.n + (size_t)re.col * Z + vo] + kLn2 * __uint_as_float(fbits(mag) ^ sk);
@@ -222,7 +226,7 @@ __device__ __noinline__ void soft_deg1(const Table &T, const Work &W, int f, int
 // and reports whether the staged rows arrived. Thread tid < nt owns checks
 // i0 + c nt + tid. FUSE: also add each message's change to its node's
 // posterior (row groups that touch every node at most once, cn_group_kernel).
-template <int NH, int ND, int MODE, typename M, int NT, bool FUSE, typename Wait>
+template <int NH, int ND, int MODE, typename M, int NT, bool SOFT, bool FUSE, typename Wait>
 __device__ __forceinline__ bool cn_compute(const Table &T, const Work &W, int f, int r, int rp, int t,
                                            int i0, const int *oa, const int *ob, const int *s_off,
                                            const float *stage, const uint32_t *sy0, int b0, Wait wait) {
@@ -236,8 +240,8 @@ __device__ __forceinline__ bool cn_compute(const Table &T, const Work &W, int f,
     const int nt = NT ? NT : (int)blockDim.x;  // threads: a multiple of 32, at most kCnThreads
     const int ws = nt >> 5;                    // decision words per check slot
     const int tid = threadIdx.x;
-    const size_t bstride = (size_t)T.n_d1 * ZW;
-    M *msg = static_cast<M *>(W.msg) + (t & 1) * W.msg_buf + (size_t)f * T.n_h * Z;
+    const size_t bstride = W.bit_f;
+    M *msg = static_cast<M *>(W.msg) + (t & 1) * W.msg_buf + (size_t)f * W.msg_f;
 
     // Per-row pointers for this thread's first check; check c sits at
     // + c * nt elements (or + c * ws words).
@@ -276,28 +280,31 @@ __device__ __forceinline__ bool cn_compute(const Table &T, const Work &W, int f,
         }
     }
     // accumulator of heavy entry k for this thread's check c: accb + oa[k] + c nt
-    int32_t *accb = W.acc + (size_t)f * T.n_hcols * 2 * Z + i0 + tid;
+    int32_t *accb = W.acc + (size_t)f * W.col_f + i0 + tid;
     const bool accum = !FUSE && W.accum != 0;
-    [[maybe_unused]] float *const Lb = W.L + (size_t)f * T.n_hcols * 2 * Z + i0 + tid;
+    [[maybe_unused]] float *const Lb = W.L + (size_t)f * W.col_f + i0 + tid;
     [[maybe_unused]] int sh[NHa];
     if constexpr (FUSE) {
 #pragma unroll
         for (int k = 0; k < NH; k++) sh[k] = oa[k] % (2 * Z);
     }
     // syndrome words of the owned checks (check c of this thread sits c * ws
-    // words after the first), loaded while the copies are in flight
-    const int sb = b0 + tid;
-    const uint32_t *sy = sy0 + (sb >> 5);
-    const int ssh = 31 - (sb & 31);
+    // words after the first), loaded while the copies are in flight; rows
+    // with a degree-1 node have the bit folded into its sign (syn_folded)
+    constexpr bool kSyn = !syn_folded(ND);
     const int dsh = 31 - (tid & 31);
     const bool lane0 = (tid & 31) == 0;
     uint32_t sw[kTmaVpt];
+    const int sb = b0 + tid;
+    const uint32_t *sy = sy0 + (sb >> 5);
+    const int ssh = 31 - (sb & 31);
 #pragma unroll
     for (int c = 0; c < kTmaVpt; c++)
-        sw[c] = i0 + c * nt + tid < Z ? (__ldg(sy + c * ws) << ssh) : 0u;
+        sw[c] = !kSyn ? 0u : i0 + c * nt + tid < Z ? (__ldg(sy + c * ws) << ssh) : 0u;
 
     const bool staged = wait();
     bool bad = false;
+    [[maybe_unused]] uint32_t badw = 0;  // sign bit: some owned check of iteration t - 1 failed
     if (staged) {
       if constexpr (QCLDPC_CN_PAIR && kTmaVpt % 2 == 0) {
         // Two checks (c, c + 1) per step, their arithmetic in packed FP32x2
@@ -323,7 +330,8 @@ __device__ __forceinline__ bool cn_compute(const Table &T, const Work &W, int f,
                     pa ^= pB[k][c * ws] << dsh;
                     pb ^= pB[k][(c + 1) * ws] << dsh;
                 }
-                bad |= (va && (pa & kSign) != 0) || (vb && (pb & kSign) != 0);
+                if (va) badw |= pa;
+                if (vb) badw |= pb;
             }
             if constexpr (kUpdate) {
 #pragma unroll
@@ -388,15 +396,15 @@ __device__ __forceinline__ bool cn_compute(const Table &T, const Work &W, int f,
                         red_add_if(accb + (oa[k] + (c + 1) * nt), acc_value(eb, W), ab);
                     } else {
                         const float2 ex = make_float2(fmaxf(s2.x, W.xmin), fmaxf(s2.y, W.xmin));
-                        const uint32_t da = ex.x < phi[k].x ? ska : (sga[k] & kSign);
-                        const uint32_t db = ex.y < phi[k].y ? skb : (sgb[k] & kSign);
-                        const uint32_t wa = __ballot_sync(0xffffffffu, va && da != 0);
-                        const uint32_t wb = __ballot_sync(0xffffffffu, vb && db != 0);
+                        const uint32_t da = ex.x < phi[k].x ? sta ^ sga[k] : sga[k];
+                        const uint32_t db = ex.y < phi[k].y ? stb ^ sgb[k] : sgb[k];
+                        const uint32_t wa = __ballot_sync(0xffffffffu, va && (int)da < 0);
+                        const uint32_t wb = __ballot_sync(0xffffffffu, vb && (int)db < 0);
                         st_if(oB[k - NH] + c * ws, wa, lane0 && va);
                         st_if(oB[k - NH] + (c + 1) * ws, wb, lane0 && vb);
-                        if (W.soft) {
-                            if (va) soft_deg1(T, W, f, t, rp + k, ia, ex.x, ska);
-                            if (vb) soft_deg1(T, W, f, t, rp + k, ib, ex.y, skb);
+                        if constexpr (SOFT) {
+                            if (va) soft_deg1(T, W, f, r, t, rp + k, ia, ex.x, ska);
+                            if (vb) soft_deg1(T, W, f, r, t, rp + k, ib, ex.y, skb);
                         }
                     }
                 }
@@ -460,17 +468,17 @@ __device__ __forceinline__ bool cn_compute(const Table &T, const Work &W, int f,
                         const uint32_t dbits = ex < phi[k] ? sk : (sg[k] & kSign);
                         const uint32_t word = __ballot_sync(0xffffffffu, valid && dbits != 0);
                         if (lane0 && valid) oB[k - NH][c * ws] = word;
-                        if (W.soft && valid) soft_deg1(T, W, f, t, rp + k, i, ex, sk);
+                        if (SOFT && valid) soft_deg1(T, W, f, r, t, rp + k, i, ex, sk);
                     }
                 }
             }
         }
       }
     }
-    return bad;
+    return bad || (int)badw < 0;
 }
 
-template <int NH, int ND, int MODE, typename M, int NT, bool FUSE>
+template <int NH, int ND, int MODE, typename M, int NT, bool SOFT, bool FUSE>
 __device__ __forceinline__ bool cn_tile(const Table &T, const Work &W, int f, int r, int rp, int t,
                                         const qc::RowDesc *dp, unsigned char *smem) {
     constexpr int NHa = NH > 0 ? NH : 1;
@@ -488,18 +496,18 @@ __device__ __forceinline__ bool cn_tile(const Table &T, const Work &W, int f, in
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
     int *s_off = reinterpret_cast<int *>(smem + 16);  // per staged row: start of its data
     float *stage = reinterpret_cast<float *>(smem + kSmemHeader);
-    const size_t bstride = (size_t)T.n_d1 * ZW;
+    const size_t bstride = W.bit_f;
     // messages of iteration t-1 (read); layered decoding writes those of t
     // to the other buffer
-    const M *msg_rd = static_cast<const M *>(W.msg) + ((t - 1) & 1) * W.msg_buf + (size_t)f * T.n_h * Z;
+    const M *msg_rd = static_cast<const M *>(W.msg) + ((t - 1) & 1) * W.msg_buf + (size_t)f * W.msg_f;
 
     // Thread 0: arm the barrier, publish each staged row's read offset
     // (row slot * (tile + 4) + 16-byte remainder), then issue the copies.
     // Staged rows: NH posteriors, NH old messages (kReadMsg), ND psi values
     // (kUpdate), then ND decision-word rows of tile / 32 + 4 words (kTest).
     if (tid == 0) {
-        const float *L = W.L + (size_t)f * T.n_hcols * 2 * Z;
-        const float *phiq = W.phiq + (size_t)f * T.n_d1 * Z;
+        const float *L = W.L + (size_t)f * W.col_f;
+        const float *phiq = W.phiq + (size_t)f * W.d1_f;
         const uint32_t *bprev = W.bits + ((size_t)((t - 1) & 1) * W.n_frames + f) * bstride;
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -546,7 +554,7 @@ __device__ __forceinline__ bool cn_tile(const Table &T, const Work &W, int f, in
     __syncthreads();  // barrier initialised, offsets published
 
     const int cb0 = r * Z + i0;
-    const bool bad = cn_compute<NH, ND, MODE, M, NT, FUSE>(
+    const bool bad = cn_compute<NH, ND, MODE, M, NT, SOFT, FUSE>(
         T, W, f, r, rp, t, i0, oa, ob, s_off, stage, W.syn + (size_t)f * W.words_m + (cb0 >> 5), cb0 & 31,
         [&] { return stage_wait(bar, W); });
     __syncthreads();
@@ -554,18 +562,18 @@ __device__ __forceinline__ bool cn_tile(const Table &T, const Work &W, int f, in
     return bad;
 }
 
-template <int MODE, typename M, int NT, bool FUSE = false>
+template <int MODE, typename M, int NT, bool SOFT, bool FUSE = false>
 __device__ __forceinline__ bool cn_tile_dispatch(const Table &T, const Work &W, int f, int r, int t,
                                                  int rp, int nh, int nd, const qc::RowDesc *dp,
                                                  unsigned char *smem) {
     switch (nh * 4 + nd) {
-        case 1 * 4 + 1: return cn_tile<1, 1, MODE, M, NT, FUSE>(T, W, f, r, rp, t, dp, smem);
-        case 2 * 4 + 0: return cn_tile<2, 0, MODE, M, NT, FUSE>(T, W, f, r, rp, t, dp, smem);
-        case 2 * 4 + 1: return cn_tile<2, 1, MODE, M, NT, FUSE>(T, W, f, r, rp, t, dp, smem);
-        case 3 * 4 + 0: return cn_tile<3, 0, MODE, M, NT, FUSE>(T, W, f, r, rp, t, dp, smem);
-        case 3 * 4 + 1: return cn_tile<3, 1, MODE, M, NT, FUSE>(T, W, f, r, rp, t, dp, smem);
-        case 4 * 4 + 0: return cn_tile<4, 0, MODE, M, NT, FUSE>(T, W, f, r, rp, t, dp, smem);
-        case 4 * 4 + 1: return cn_tile<4, 1, MODE, M, NT, FUSE>(T, W, f, r, rp, t, dp, smem);
+        case 1 * 4 + 1: return cn_tile<1, 1, MODE, M, NT, SOFT, FUSE>(T, W, f, r, rp, t, dp, smem);
+        case 2 * 4 + 0: return cn_tile<2, 0, MODE, M, NT, SOFT, FUSE>(T, W, f, r, rp, t, dp, smem);
+        case 2 * 4 + 1: return cn_tile<2, 1, MODE, M, NT, SOFT, FUSE>(T, W, f, r, rp, t, dp, smem);
+        case 3 * 4 + 0: return cn_tile<3, 0, MODE, M, NT, SOFT, FUSE>(T, W, f, r, rp, t, dp, smem);
+        case 3 * 4 + 1: return cn_tile<3, 1, MODE, M, NT, SOFT, FUSE>(T, W, f, r, rp, t, dp, smem);
+        case 4 * 4 + 0: return cn_tile<4, 0, MODE, M, NT, SOFT, FUSE>(T, W, f, r, rp, t, dp, smem);
+        case 4 * 4 + 1: return cn_tile<4, 1, MODE, M, NT, SOFT, FUSE>(T, W, f, r, rp, t, dp, smem);
         default: return false;
     }
 }
@@ -575,7 +583,7 @@ __device__ __forceinline__ bool cn_tile_dispatch(const Table &T, const Work &W, 
 // row, frame) with blocks of cn_launch's thread count, dynamic shared memory
 // sized by cn_launch for the code's widest exact-shape row. Rows of other
 // shapes take the generic path.
-template <int MAXD, typename M, int NT>
+template <int MAXD, typename M, int NT, bool SOFT>
 __global__ void __launch_bounds__(kCnThreads, NT ? QCLDPC_CN_TMA_MINBLOCKS : QCLDPC_CN_FIT_MINBLOCKS)
     cn_tma_kernel(const __grid_constant__ Table T, const __grid_constant__ Work W) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -610,10 +618,10 @@ __global__ void __launch_bounds__(kCnThreads, NT ? QCLDPC_CN_TMA_MINBLOCKS : QCL
     bool bad;
     if (exact_shape(nh, nd)) {
         switch (mode) {
-            case kFirst: bad = cn_tile_dispatch<kFirst, M, NT>(T, W, f, r, t, rp, nh, nd, dp, smem); break;
-            case kSteady: bad = cn_tile_dispatch<kSteady, M, NT>(T, W, f, r, t, rp, nh, nd, dp, smem); break;
-            case kSteadyTest: bad = cn_tile_dispatch<kSteadyTest, M, NT>(T, W, f, r, t, rp, nh, nd, dp, smem); break;
-            default: bad = cn_tile_dispatch<kTestOnly, M, NT>(T, W, f, r, t, rp, nh, nd, dp, smem); break;
+            case kFirst: bad = cn_tile_dispatch<kFirst, M, NT, SOFT>(T, W, f, r, t, rp, nh, nd, dp, smem); break;
+            case kSteady: bad = cn_tile_dispatch<kSteady, M, NT, SOFT>(T, W, f, r, t, rp, nh, nd, dp, smem); break;
+            case kSteadyTest: bad = cn_tile_dispatch<kSteadyTest, M, NT, SOFT>(T, W, f, r, t, rp, nh, nd, dp, smem); break;
+            default: bad = cn_tile_dispatch<kTestOnly, M, NT, SOFT>(T, W, f, r, t, rp, nh, nd, dp, smem); break;
         }
     } else {
         bad = cn_row_generic<MAXD, M>(T, W, f, r, t, mode, blockIdx.x * blockDim.x * kTmaVpt + threadIdx.x,
@@ -633,7 +641,7 @@ __global__ void __launch_bounds__(kCnThreads, NT ? QCLDPC_CN_TMA_MINBLOCKS : QCL
 // the schedule: with this kernel for 30 of the 49 rows and programmatic edges
 // between all of them, four iterations of the 49-group schedule on 16 frames of
 // n = 10^6 went from 2.66 to 2.32 ms.
-template <typename M>
+template <typename M, bool SOFT>
 __global__ void __launch_bounds__(kCnThreads, QCLDPC_CN_FIT_MINBLOCKS)
     cn_group_kernel(const __grid_constant__ Table T, const __grid_constant__ Work W) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -645,30 +653,35 @@ __global__ void __launch_bounds__(kCnThreads, QCLDPC_CN_FIT_MINBLOCKS)
     const int4 head = __ldg(reinterpret_cast<const int4 *>(dp));  // r, rp, nh, nd
     const int t = W.t[f] - 1;
     if (t == 1)
-        cn_tile_dispatch<kFirst, M, 0, true>(T, W, f, head.x, t, head.y, head.z, head.w, dp, smem);
+        cn_tile_dispatch<kFirst, M, 0, SOFT, true>(T, W, f, head.x, t, head.y, head.z, head.w, dp, smem);
     else
-        cn_tile_dispatch<kSteady, M, 0, true>(T, W, f, head.x, t, head.y, head.z, head.w, dp, smem);
+        cn_tile_dispatch<kSteady, M, 0, SOFT, true>(T, W, f, head.x, t, head.y, head.z, head.w, dp, smem);
+}
+
+template <typename M, bool SOFT>
+void *cn_kernel_pick(int maxdeg, int nt) {
+    if (nt < 0) return (void *)cn_group_kernel<M, SOFT>;
+    if (nt == kCnThreads) {
+        if (maxdeg <= 5) return (void *)cn_tma_kernel<5, M, kCnThreads, SOFT>;
+        if (maxdeg <= 8) return (void *)cn_tma_kernel<8, M, kCnThreads, SOFT>;
+        return (void *)cn_tma_kernel<16, M, kCnThreads, SOFT>;
+    }
+    if (maxdeg <= 5) return (void *)cn_tma_kernel<5, M, 0, SOFT>;
+    if (maxdeg <= 8) return (void *)cn_tma_kernel<8, M, 0, SOFT>;
+    return (void *)cn_tma_kernel<16, M, 0, SOFT>;
 }
 
 template <typename M>
-void *cn_kernel_select(int maxdeg, int nt) {
-    if (nt < 0) return (void *)cn_group_kernel<M>;
-    if (nt == kCnThreads) {
-        if (maxdeg <= 5) return (void *)cn_tma_kernel<5, M, kCnThreads>;
-        if (maxdeg <= 8) return (void *)cn_tma_kernel<8, M, kCnThreads>;
-        return (void *)cn_tma_kernel<16, M, kCnThreads>;
-    }
-    if (maxdeg <= 5) return (void *)cn_tma_kernel<5, M, 0>;
-    if (maxdeg <= 8) return (void *)cn_tma_kernel<8, M, 0>;
-    return (void *)cn_tma_kernel<16, M, 0>;
+void *cn_kernel_select(int maxdeg, int nt, bool soft) {
+    return soft ? cn_kernel_pick<M, true>(maxdeg, nt) : cn_kernel_pick<M, false>(maxdeg, nt);
 }
 
 template <typename M>
 void cn_raise_smem_cap(int cap) {
-    const void *k[] = {(const void *)cn_tma_kernel<5, M, kCnThreads>, (const void *)cn_tma_kernel<8, M, kCnThreads>,
-                       (const void *)cn_tma_kernel<16, M, kCnThreads>, (const void *)cn_tma_kernel<5, M, 0>,
-                       (const void *)cn_tma_kernel<8, M, 0>, (const void *)cn_tma_kernel<16, M, 0>,
-                       (const void *)cn_group_kernel<M>};
-    for (const void *f : k) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
+    for (int soft = 0; soft < 2; soft++)
+        for (int maxdeg : {5, 8, 16})
+            for (int nt : {-1, 0, kCnThreads})
+                cudaFuncSetAttribute(cn_kernel_select<M>(maxdeg, nt, soft != 0),
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
 }
 }  // namespace

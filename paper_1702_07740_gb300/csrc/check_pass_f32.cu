@@ -2,6 +2,6 @@
 #include "check_pass.cuh"
 
 namespace qc {
-void *cn_kernel_f32(int maxdeg, int nt) { return cn_kernel_select<float>(maxdeg, nt); }
+void *cn_kernel_f32(int maxdeg, int nt, bool soft) { return cn_kernel_select<float>(maxdeg, nt, soft); }
 void cn_smem_cap_f32(int cap) { cn_raise_smem_cap<float>(cap); }
 }  // namespace qc

@@ -78,7 +78,7 @@ namespace {
 // ------------------------------------------------------------ kernels
 
 // Initial state: L = Q (heavy), phiq = +-Phi(|clip Q|) and the iteration-0
-// decisions of the degree-1 nodes, frame flags, loop counter t = 1.
+// decisions of the degree-1 nodes (syndrome folded in), frame flags, loop counter t = 1.
 // The message arrays need no initialisation: iteration 1 reads m = 0.
 __global__ void __launch_bounds__(kThreads) init_kernel(const __grid_constant__ Table T,
                                                         const __grid_constant__ Work W) {
@@ -118,9 +118,11 @@ __global__ void __launch_bounds__(kThreads) init_kernel(const __grid_constant__ 
             const float a = fmaxf(fminf(fabsf(qv) * kLog2e, W.clip), W.xmin);
             const float p = psi_f(a);
             const size_t off = ((size_t)f * T.n_d1 + k) * Z + i;
-            W.phiq[off] = qv < 0.0f ? -p : p;
-            if (W.soft) W.post1[off] = qv;  // iteration-0 posterior, buffer 0
             neg = qv < 0.0f;
+            const int r = T.d1_row[k];
+            if (row_syn_folded(T, r)) neg ^= syn_sign(W, f, r * Z + i) != 0;
+            W.phiq[off] = neg ? -p : p;
+            if (W.soft) W.post1[off] = qv;  // iteration-0 posterior, buffer 0
         }
         const uint32_t word = __ballot_sync(0xffffffffu, neg);
         if (lane == 0) W.bits[((size_t)f * T.n_d1 + k) * W.ZW + wd] = word;
@@ -488,6 +490,8 @@ __global__ void __launch_bounds__(kThreads) final_kernel(const __grid_constant__
                 const uint32_t word =
                     W.bits[(((size_t)b * W.n_frames + f) * T.n_d1 + d) * W.ZW + (i >> 5)];
                 dec = (word >> (i & 31)) & 1u;
+                const int r = T.d1_row[d];
+                if (row_syn_folded(T, r)) dec ^= syn_sign(W, f, r * Z + i) != 0;
             }
         }
         const uint32_t word = __ballot_sync(0xffffffffu, dec);
@@ -626,10 +630,11 @@ int sm_count() {
 
 // The check-pass kernel for a message format (its translation unit): full
 // kThreads-thread blocks, or blocks of any width (nt < kThreads).
-void *cn_tma_kernel_for(int maxdeg, int fmt, int nt) {
-    if (fmt == 1) return qc::cn_kernel_f16(maxdeg, nt);
-    if (fmt == 2) return qc::cn_kernel_i8(maxdeg, nt);
-    return qc::cn_kernel_f32(maxdeg, nt);
+void *cn_tma_kernel_for(int maxdeg, const Work &w, int nt) {
+    const bool soft = w.soft != 0;
+    if (w.fmt == 1) return qc::cn_kernel_f16(maxdeg, nt, soft);
+    if (w.fmt == 2) return qc::cn_kernel_i8(maxdeg, nt, soft);
+    return qc::cn_kernel_f32(maxdeg, nt, soft);
 }
 
 void *lvn_kernel_for(int fmt) {
@@ -739,15 +744,15 @@ int cn_threads(int Z) {
 
 // nt_set (non-zero) overrides the block width (qcldpc_params cn_threads);
 // a check's arithmetic does not depend on it.
-CnLaunch cn_launch(const Table &T, int F, int fmt, int nt_set = 0) {
+CnLaunch cn_launch(const Table &T, const Work &w, int nt_set) {
     CnLaunch c;
     {
         const int nt = nt_set ? nt_set : cn_threads(T.Z), tile = nt * kTmaVpt;
         // the code's widest exact-shape row (its staged rows and word rows)
         const size_t smem = kSmemHeader + (size_t)T.stage_rows_max * (tile + 4) * 4 +
                             (size_t)T.stage_words_max * (tile / 32 + 4) * 4;
-        c.func = cn_tma_kernel_for(T.max_row_deg, fmt, nt);
-        c.grid = dim3((unsigned)((T.Z + tile - 1) / tile), (unsigned)T.mb, (unsigned)F);
+        c.func = cn_tma_kernel_for(T.max_row_deg, w, nt);
+        c.grid = dim3((unsigned)((T.Z + tile - 1) / tile), (unsigned)T.mb, (unsigned)w.n_frames);
         c.block = dim3((unsigned)nt);
         c.smem = smem;
         // Capacity for the largest staged row set (4 heavy + 1 degree-1).
@@ -838,7 +843,7 @@ cudaError_t add_loop_body(cudaGraph_t body, const qcldpc_code *code, const Work 
     qc::ColsInline ccopy = code->cols_in;
     void *args[] = {&tcopy, &wcopy};
     void *vn_args[] = {&tcopy, &wcopy, &ccopy};
-    const CnLaunch cl = cn_launch(T, F, w0.fmt, w0.cn_nt);
+    const CnLaunch cl = cn_launch(T, w0, w0.cn_nt);
     cudaError_t err;
     if (w0.layered) wcopy.pass = kPassTest;
     void *ctrl_args[] = {&wcopy, &handle};
@@ -887,7 +892,7 @@ cudaError_t add_loop_body(cudaGraph_t body, const qcldpc_code *code, const Work 
             grid.y = (unsigned)wg.lrows;
             cudaGraphNode_t a, b;
             const bool fuse = group_fuses(code, wg.lrow0, wg.lrow0 + wg.lrows);
-            if ((err = add_kernel(&a, body, &prev, 1, fuse ? cn_tma_kernel_for(T.max_row_deg, w0.fmt, -1) : cl.func,
+            if ((err = add_kernel(&a, body, &prev, 1, fuse ? cn_tma_kernel_for(T.max_row_deg, w0, -1) : cl.func,
                                   grid, cl.block, gargs, cl.smem, true)) != cudaSuccess)
                 return err;
             if (fuse) {
@@ -949,7 +954,7 @@ int stream_decode(qcldpc_code *code, const Work &w, cudaStream_t stream) {
     const int F = w.n_frames;
     const int blocks = sm_count() * 4;
     init_kernel<<<blocks, kThreads, 0, stream>>>(T, w);
-    const CnLaunch cl = cn_launch(T, F, w.fmt, w.cn_nt);
+    const CnLaunch cl = cn_launch(T, w, w.cn_nt);
     Table tcopy = T;
     Work wcopy = w;
     if (w.layered) wcopy.pass = kPassTest;
@@ -987,7 +992,7 @@ int stream_decode(qcldpc_code *code, const Work &w, cudaStream_t stream) {
             dim3 grid = cl.grid;
             grid.y = (unsigned)wg.lrows;
             const bool fuse = fuses[g];
-            err = cudaLaunchKernel(fuse ? cn_tma_kernel_for(T.max_row_deg, w.fmt, -1) : cl.func, grid, cl.block, gargs,
+            err = cudaLaunchKernel(fuse ? cn_tma_kernel_for(T.max_row_deg, w, -1) : cl.func, grid, cl.block, gargs,
                                    cl.smem, stream);
             if (err == cudaSuccess && !fuse)
                 err = cudaLaunchKernel(lvn_kernel_for(w.fmt), vn_grid(T, F), dim3(kThreads), gargs,
@@ -1002,6 +1007,16 @@ int stream_decode(qcldpc_code *code, const Work &w, cudaStream_t stream) {
     if (err != cudaSuccess) return qc::cuda_fail(err, "decode (stream mode): launch");
     qc::clear_error();
     return QCLDPC_OK;
+}
+
+// Per-frame strides of the workspace arrays (their offsets fit int32, see
+// Table), and the decision words of a row.
+void set_strides(const Table &T, Work &w) {
+    w.ZW = (T.Z + 31) / 32;
+    w.msg_f = (uint32_t)((size_t)T.n_h * T.Z);
+    w.col_f = (uint32_t)((size_t)T.n_hcols * 2 * T.Z);
+    w.d1_f = (uint32_t)((size_t)T.n_d1 * T.Z);
+    w.bit_f = (uint32_t)((size_t)T.n_d1 * w.ZW);
 }
 
 // The kernels' argument block for one decode call of `code` on F frames
@@ -1037,7 +1052,7 @@ Work make_work(const qcldpc_code *code, const qcldpc_params &p, int F, int max_i
     w.max_iter = max_iter;
     w.et_start = p.et_start;
     w.soft = soft ? 1 : 0;
-    w.ZW = (T.Z + 31) / 32;
+    set_strides(T, w);
     w.clip = p.clip > 0.0f ? p.clip * kLog2e : INFINITY;  // base-2 units
     w.xmin = p.phi_floor * kLog2e;
     w.xmin_h = heavy_out_floor(w.clip, w.xmin);
@@ -1551,7 +1566,7 @@ extern "C" int qcldpc_autotune_shapes(const qcldpc_code *code_c, int n_frames, v
     float tc[kNc], tv[kNv];
     int bc = 0, bv = 0;
     for (int i = 0; i < kNc; i++) {
-        const CnLaunch cl = cn_launch(T, n_frames, w.fmt, 32 * (i + 1));
+        const CnLaunch cl = cn_launch(T, w, 32 * (i + 1));
         tc[i] = time(cl.func, cl.grid, cl.block, args, cl.smem);
         if (tc[i] < tc[bc]) bc = i;
     }
@@ -1599,7 +1614,7 @@ extern "C" int qcldpc_time_passes(const qcldpc_code *code_c, int n_frames, void 
         if ((err = cudaEventCreate(&ev[i])) != cudaSuccess) return cuda_fail(err, "time_passes: cudaEventCreate");
     const Table &T = code->tab;
     replay_prep_kernel<<<1, 256, 0, stream>>>(w);
-    const CnLaunch cl = cn_launch(T, n_frames, w.fmt, w.cn_nt);
+    const CnLaunch cl = cn_launch(T, w, w.cn_nt);
     Table tcopy = T;
     void *args[] = {&tcopy, &w};
     cudaEventRecord(ev[0], stream);
@@ -1707,8 +1722,10 @@ __global__ void __launch_bounds__(kThreads) pool_load_kernel(const __grid_consta
             const float qv = llr_src[q * N + (int64_t)T.d1_col[k] * Z + vo];
             const float a = fmaxf(fminf(fabsf(qv) * kLog2e, W.clip), W.xmin);
             const float p = psi_f(a);
-            W.phiq[((size_t)f * T.n_d1 + k) * Z + i] = qv < 0.0f ? -p : p;
             neg = qv < 0.0f;
+            const int r = T.d1_row[k], c = r * Z + i;
+            if (row_syn_folded(T, r)) neg ^= (syn_src[q * W.words_m + (c >> 5)] >> (c & 31)) & 1u;
+            W.phiq[((size_t)f * T.n_d1 + k) * Z + i] = neg ? -p : p;
         }
         const uint32_t word = __ballot_sync(0xffffffffu, neg);
         if (lane == 0) {
@@ -1754,6 +1771,8 @@ __global__ void __launch_bounds__(kThreads) pool_collect_kernel(
                 const uint32_t word =
                     W.bits[(((size_t)b * W.n_frames + f) * T.n_d1 + d) * W.ZW + (i >> 5)];
                 dec = (word >> (i & 31)) & 1u;
+                const int r = T.d1_row[d];
+                if (row_syn_folded(T, r)) dec ^= syn_sign(W, f, r * Z + i) != 0;
             }
         }
         const uint32_t word = __ballot_sync(0xffffffffu, dec);
@@ -1831,7 +1850,7 @@ cudaError_t add_pool_passes(cudaGraph_t g, const qcldpc_pool *pool, int n_passes
     void *vn_args[] = {&tcopy, &wcopy, &ccopy};
     cudaGraphConditionalHandle none = 0;
     void *ctrl_args[] = {&wcopy, &none};
-    const CnLaunch cl = cn_launch(T, F, pool->w.fmt, pool->w.cn_nt);
+    const CnLaunch cl = cn_launch(T, pool->w, pool->w.cn_nt);
     const VnLaunch vl = vn_launch(T, F, pool->w.fmt, pool->w.vn_vpt, pool->w.vn_split);
     const bool layered = pool->w.layered != 0;
     if (layered) wcopy.pass = kPassTest;
@@ -1883,7 +1902,7 @@ cudaError_t add_pool_passes(cudaGraph_t g, const qcldpc_pool *pool, int n_passes
             grid.y = (unsigned)wg[k].lrows;
             cudaGraphNode_t x, y;
             const bool fuse = fuses[k];
-            err = add_kernel(&x, g, &prev, 1, fuse ? cn_tma_kernel_for(T.max_row_deg, pool->w.fmt, -1) : cl.func,
+            err = add_kernel(&x, g, &prev, 1, fuse ? cn_tma_kernel_for(T.max_row_deg, pool->w, -1) : cl.func,
                              grid, cl.block, gargs, cl.smem, true);
             y = x;
             if (err == cudaSuccess && !fuse)
@@ -1971,7 +1990,7 @@ extern "C" int qcldpc_pool_create(const qcldpc_code *code_c, int n_slots, int ma
     w.n_frames = n_slots;
     w.max_iter = max_iter;
     w.et_start = p.et_start;
-    w.ZW = (code->tab.Z + 31) / 32;
+    set_strides(code->tab, w);
     w.clip = p.clip > 0.0f ? p.clip * kLog2e : INFINITY;
     w.xmin = p.phi_floor * kLog2e;
     w.xmin_h = heavy_out_floor(w.clip, w.xmin);

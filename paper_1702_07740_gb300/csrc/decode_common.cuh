@@ -139,10 +139,11 @@ struct Work {
     void *msg;             // [F][n_h][Z] messages in the storage format fmt (layered:
                            // two such buffers msg_buf elements apart, by iteration parity)
     float *L;              // [F][n_hcols][2Z]
-    float *phiq;           // [F][n_d1][Z]
-    uint32_t *bits;        // [2][F][n_d1][ZW]
+    float *phiq;           // [F][n_d1][Z] (signs: see syn_folded)
+    uint32_t *bits;        // [2][F][n_d1][ZW] (see syn_folded)
     float *post1;          // [2][F][n_d1][Z] (soft output only)
     int64_t n, words_m, words_k;
+    uint32_t msg_f, col_f, d1_f, bit_f;  // elements of one frame: n_h Z, 2Z n_hcols, n_d1 Z, n_d1 ZW
     int32_t n_frames, max_iter, et_start, soft, ZW, fmt;
     float clip, xmin;      // base-2 units
     float xmin_h;          // floor of a heavy output's exclusive sum: max(xmin, psi(clip)),
@@ -312,6 +313,24 @@ __device__ __forceinline__ void load_offsets(const qc::RowDesc *dp, int (&oa)[qc
 }
 __device__ __forceinline__ uint32_t fbits(float x) { return __float_as_uint(x); }
 
+// Syndrome bit of check c (row * Z + offset) of frame f, as a sign bit.
+__device__ __forceinline__ uint32_t syn_sign(const Work &W, int64_t f, int c) {
+    return __ldg(W.syn + f * W.words_m + (c >> 5)) << (31 - (c & 31)) & kSign;
+}
+
+// A check with one degree-1 neighbour p keeps its syndrome bit folded into
+// that neighbour: phiq holds psi(|Q_p|) with the sign of Q_p times the
+// syndrome sign, and `bits` the decision C_p plus (mod 2) the syndrome bit.
+// The sign total of the check, its parity and the choice between sgn(m_cp)
+// and sgn(Q_p) then come out without the check pass ever reading the
+// syndrome (one unaligned load, a range test and a shift per check less);
+// outputs of degree-1 nodes take the bit out again. nd: the row's degree-1
+// circulants.
+__host__ __device__ constexpr bool syn_folded(int nd) { return nd == 1; }
+__device__ __forceinline__ bool row_syn_folded(const Table &T, int r) {
+    return syn_folded(T.row_ptr[r + 1] - T.row_ptr[r] - T.row_nh[r]);
+}
+
 // Storage formats of the check-to-variable messages (computation is FP32):
 // FP32, FP16 (round to nearest), or int8 codes q with m = q * qstep,
 // |q| <= 127 (values beyond saturate; the quantum is one scale for the one
@@ -393,10 +412,11 @@ namespace qc {
 // Check-pass kernels of one storage format (FP32, FP16, int8) for codes whose
 // rows have at most maxdeg circulants: the full-block kernel when nt ==
 // kCnThreads, the one that updates a row group's posteriors too when nt < 0,
-// else the one that takes its width from the launch.
-void *cn_kernel_f32(int maxdeg, int nt);
-void *cn_kernel_f16(int maxdeg, int nt);
-void *cn_kernel_i8(int maxdeg, int nt);
+// else the one that takes its width from the launch; with degree-1 posteriors
+// (soft) or without.
+void *cn_kernel_f32(int maxdeg, int nt, bool soft);
+void *cn_kernel_f16(int maxdeg, int nt, bool soft);
+void *cn_kernel_i8(int maxdeg, int nt, bool soft);
 // Raise the dynamic shared-memory cap of that format's check-pass kernels.
 void cn_smem_cap_f32(int cap);
 void cn_smem_cap_f16(int cap);

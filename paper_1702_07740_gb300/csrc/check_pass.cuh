@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(kCnThreads, NT ? QCLDPC_CN_TMA_MINBLOCKS : QCL
                                       kTmaVpt, (int)blockDim.x);
     }
     if (mode == kSteadyTest || mode == kTestOnly) {
-        if (__syncthreads_or(bad) && threadIdx.x == 0) W.fail[f] = t;
+        if (__syncthreads_or(bad) && threadIdx.x == 0) W.fail[(size_t)f * W.fail_f] = t;
     }
 }
 

@@ -134,7 +134,8 @@ struct Work {
     int32_t *state;        // [F] slot state for pools (0 free, 1 running, 2 stopped) or null
     int32_t *active;       // [F]
     int32_t *ct;           // [F] iteration the current flooding check pass runs, 0: frame not running
-    int32_t *fail;         // [F] iteration of the last pass whose stop test failed (0: none yet)
+    int32_t *fail;         // [F], fail_f words apart: iteration of the last pass whose stop test
+                           // failed (0: none yet)
     int32_t *err;          // device error word (a bounded wait gave up)
     void *msg;             // [F][n_h][Z] messages in the storage format fmt (layered:
                            // two such buffers msg_buf elements apart, by iteration parity)
@@ -143,6 +144,7 @@ struct Work {
     uint32_t *bits;        // [2][F][n_d1][ZW] (see syn_folded)
     float *post1;          // [2][F][n_d1][Z] (soft output only)
     int64_t n, words_m, words_k;
+    int32_t fail_f;
     uint32_t msg_f, col_f, d1_f, bit_f;  // elements of one frame: n_h Z, 2Z n_hcols, n_d1 Z, n_d1 ZW
     int32_t n_frames, max_iter, et_start, soft, ZW, fmt;
     float clip, xmin;      // base-2 units

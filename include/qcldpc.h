@@ -187,8 +187,8 @@ typedef struct qcldpc_params {
     /* Launch shapes; 0 (default) lets the library choose. None of them
        changes a result bit (qcldpc_autotune_shapes picks them by time). */
     int32_t cn_threads;  /* threads per check-pass block: a multiple of 32,
-                            32..256; a block evaluates 4 checks per thread of
-                            one base row */
+                            32..256; a block evaluates 2 to 8 checks per thread
+                            of one base row */
     int32_t vn_nodes;    /* variable pass: heavy nodes per thread, 1..3 */
     int32_t vn_split;    /* variable pass: 1 = a thread adds both partial sums
                             of its nodes, 2 = two thread groups, one per

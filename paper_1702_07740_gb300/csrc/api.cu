@@ -303,10 +303,11 @@ extern "C" int qcldpc_create_code(int mb, int nb, int Z, int n_circ,
         H.row_order.assign(order.begin(), order.end());
     }
     // Staging footprint of the widest exact-shape row.
-    T.stage_rows_max = T.stage_words_max = 0;
+    T.stage_rows_max = T.stage_words_max = T.exact_rows = 0;
     for (int r = 0; r < mb; r++) {
         const int nh = H.row_nh[r], nd = H.row_ptr[r + 1] - H.row_ptr[r] - nh;
         if (!exact_shape(nh, nd)) continue;
+        T.exact_rows++;
         T.stage_rows_max = std::max(T.stage_rows_max, 2 * nh + nd);
         T.stage_words_max = std::max(T.stage_words_max, nd);
     }

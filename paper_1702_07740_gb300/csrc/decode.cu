@@ -20,7 +20,7 @@
 // itself (Step 4 of Algorithm 1 for degree-1 nodes).
 //
 // One iteration t is two streaming kernels:
-//   check pass  (cn_tma_kernel) per check c (row r, offset i): L_vc = clip(L_v - m_cv(t-1)) for
+//   check pass  (cn_direct_kernel or cn_tma_kernel) per check c (row r, offset i): L_vc = clip(L_v - m_cv(t-1)) for
 //               heavy neighbours v = (col, (i+s) mod Z), Phi-domain exclusive
 //               sums, m_cv(t) written back in place; decisions of the degree-1
 //               neighbours of iteration t. It also evaluates the stop test of
@@ -535,7 +535,8 @@ __global__ void replay_prep_kernel(const __grid_constant__ Work W) {
 // apart anyway, and stay packed). Far from convergence every check block
 // stores its frame's word, and packed words put all those stores into one line
 // of the L2: with lines apart an iteration of 16 frames took 99.8 us instead of
-// 101.7 (n = 10^6), and 115.8 instead of 122.7 (multi-edge code).
+// 101.7 (n = 10^6, staged check pass), and 115.8 instead of 122.7 (multi-edge
+// code).
 constexpr int kFailSpreadMax = 1024;
 constexpr int kFailLine = 32;
 int fail_stride(int F) { return F <= kFailSpreadMax ? kFailLine : 1; }
@@ -544,7 +545,6 @@ struct Layout {
     size_t t, err, active, ct, fail, msg, L, acc, phiq, bits, post1, total;
     size_t flags_extra;  // bytes of ct and of the fail words' spacing, in total
 };
-
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -754,10 +754,40 @@ int cn_threads(int Z) {
     return std::min(kCnThreads, 32 * ((per + 32 * kTmaVpt - 1) / (32 * kTmaVpt)));
 }
 
+// Checks per lane of the direct check pass (check_direct.cuh), or 0 for the
+// staged one. Direct: flooding with accumulated posteriors, every row of an
+// exact shape (its kernels have no generic row), and no test switch that makes
+// staged waits run out; a requested block width above its own takes the staged
+// pass. Eight checks per lane share a warp's set-up and overlap its loads; a
+// grid that would fill less than half of the resident warps wants more warps
+// of two. Per iteration: 16 frames of n = 10^6 99.8 us staged, 86.9 with 8;
+// one frame (3,871 warps of 8) 14.0 staged, 12.2 with 8, 13.2 with 4; 7 frames
+// of 9 rows, Z = 9,999 (1,440 a chain) 9.1 with 2, 9.9 with 4; one frame,
+// Z = 512 (98) 7.0 staged, 8.2 with 8, 5.7 with 2. Soft output, a small-batch
+// option, has the direct form for small grids only.
+int cn_direct_slots(const Table &T, const Work &w, int nt_set) {
+    if (w.layered || !w.accum || w.stall_extra || nt_set > qc::kCnDirectThreads || T.exact_rows != T.mb) return 0;
+    const long long resident = (long long)sm_count() * (kCdMinBlocks * qc::kCnDirectThreads / 32);
+    const long long warps8 = (long long)T.mb * w.n_frames * ((T.Z + 255) / 256);
+    if (2 * warps8 < resident) return 2;
+    return w.soft ? 0 : 8;
+}
+
 // nt_set (non-zero) overrides the block width (qcldpc_params cn_threads);
 // a check's arithmetic does not depend on it.
 CnLaunch cn_launch(const Table &T, const Work &w, int nt_set) {
     CnLaunch c;
+    if (const int slots = cn_direct_slots(T, w, nt_set)) {
+        const int fit = 32 * ((T.Z + 32 * slots - 1) / (32 * slots));  // warps that cover a row
+        const int nt = nt_set ? nt_set : std::min(qc::kCnDirectThreads, fit), tile = nt * slots;
+        c.func = w.fmt == 1   ? qc::cn_direct_f16(slots, w.soft != 0)
+                 : w.fmt == 2 ? qc::cn_direct_i8(slots, w.soft != 0)
+                              : qc::cn_direct_f32(slots, w.soft != 0);
+        c.grid = dim3((unsigned)((T.Z + tile - 1) / tile), (unsigned)T.mb, (unsigned)w.n_frames);
+        c.block = dim3((unsigned)nt);
+        c.smem = 0;
+        return c;
+    }
     {
         const int nt = nt_set ? nt_set : cn_threads(T.Z), tile = nt * kTmaVpt;
         // the code's widest exact-shape row (its staged rows and word rows)

@@ -104,6 +104,11 @@ constexpr int kCnUnroll = QCLDPC_CN_UNROLL;
 #ifndef QCLDPC_CN_FIT_MINBLOCKS
 #define QCLDPC_CN_FIT_MINBLOCKS QCLDPC_CN_TMA_MINBLOCKS
 #endif
+// Direct check pass: resident full blocks per SM it is compiled for.
+#ifndef QCLDPC_CD_MINBLOCKS
+#define QCLDPC_CD_MINBLOCKS 7
+#endif
+constexpr int kCdMinBlocks = QCLDPC_CD_MINBLOCKS;
 constexpr int kTile = kCnThreads * kTmaVpt;    // checks per block, at most
 constexpr int kStage = kTile + 4;              // staged floats per row (16-byte realignment)
 constexpr int kStageWords = kTile / 32 + 4;    // staged decision words per row
@@ -419,6 +424,11 @@ namespace qc {
 void *cn_kernel_f32(int maxdeg, int nt, bool soft);
 void *cn_kernel_f16(int maxdeg, int nt, bool soft);
 void *cn_kernel_i8(int maxdeg, int nt, bool soft);
+// The check pass that loads its operands directly (check_direct.cuh).
+constexpr int kCnDirectThreads = 128;
+void *cn_direct_f32(int slots, bool soft);
+void *cn_direct_f16(int slots, bool soft);
+void *cn_direct_i8(int slots, bool soft);
 // Raise the dynamic shared-memory cap of that format's check-pass kernels.
 void cn_smem_cap_f32(int cap);
 void cn_smem_cap_f16(int cap);

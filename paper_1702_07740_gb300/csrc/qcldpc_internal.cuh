@@ -70,7 +70,7 @@ struct Table {
     int32_t max_row_deg;
     int32_t stage_rows_max;   // max over exact-shape rows of 2 nh + nd (staged float rows)
     int32_t stage_words_max;  // max over exact-shape rows of nd (staged decision-word rows)
-    int32_t pad_;
+    int32_t exact_rows;       // rows of an exact shape (see exact_shape)
     const int32_t *row_ptr;    // [mb + 1] into rows[]
     const int32_t *row_nh;     // [mb] heavy entries of the row
     const int32_t *row_order;  // [mb] rows sorted by shape (check-node grid order)

@@ -3,7 +3,8 @@
 Each form is compared with the oracle or with the other form that computes
 the same bits: word-wise syndromes (rows that end inside a word, windows that
 wrap), the vector form of the d-dimensional maps (unaligned buffers, tails),
-and row groups whose check pass updates the posteriors itself.
+the check pass that loads its operands directly against the staged one, and
+row groups whose check pass updates the posteriors itself.
 """
 import numpy as np
 import pytest
@@ -67,6 +68,54 @@ def test_maps_of_any_alignment_and_tail(d, n, offset):
     assert np.all(np.abs(llr.cpu().numpy() - ref) <= 16 * U32 * (2 * snr / d) * xb * mb + 2 * U32 * np.abs(ref))
     for t in (m_all, l_all):
         assert (t[:offset] == 7.0).all() and (t[offset + n:] == 7.0).all()
+
+
+@pytest.mark.parametrize("fmt", [0, 1, 2])
+@pytest.mark.parametrize("maker, Z", [
+    (odd_code, 1), (odd_code, 5), (odd_code, 37), (synth.rate002_code, 31), (synth.rate002_code, 33),
+    (synth.rate002_code, 127), (synth.rate002_code, 129), (synth.rate002_code, 257),
+    (synth.rate005_code, 1023), (synth.rate010_code, 1025), (synth.rate002_code, 2049), (synth.met_code, 41),
+])
+def test_check_pass_forms_agree(maker, Z, fmt):
+    """Key bits, flags and stop iterations are the same whether the check pass
+    loads its operands directly or stages them (cn_threads above 128), with
+    soft output or without, in one chain or two."""
+    fr = make_frames(maker(Z), 0.12 if maker is synth.rate002_code else 0.3, 3, d=2)
+    code = q.create_code_from(fr.code_dict)
+    llr, syn = dev(fr.q64.astype(np.float32).reshape(-1)), dev(packed(fr.syn).view(np.int32).reshape(-1))
+    for max_iter, et_start in ((0, 1), (1, 1), (12, 1), (12, 13), (9, 5)):
+        out, post = [], []
+        for soft, groups, cn in ((True, 0, 0), (True, 0, 160), (False, 0, 0), (False, 1, 0), (False, 1, 32),
+                                 (False, 1, 160), (False, 2, 256)):
+            p = q.qcldpc_params_init(msg_format=fmt, et_start=et_start, frame_groups=groups, cn_threads=cn)
+            dec = q.Decoder(code, fr.F, p, soft=soft)
+            dec.decode(llr, syn, max_iter)
+            torch.cuda.synchronize()
+            out.append((dec.keys.cpu(), dec.converged.cpu(), dec.iters.cpu()))
+            post += [dec.posterior.cpu()] if soft else []
+        assert torch.equal(post[0], post[1]), (max_iter, et_start)
+        for i, o in enumerate(out[1:]):
+            assert all(torch.equal(a, b) for a, b in zip(o, out[0])), (i, max_iter, et_start)
+
+
+@pytest.mark.parametrize("fmt", [0, 1, 2])
+def test_check_pass_forms_agree_on_full_grids(fmt):
+    """24 frames at Z = 2049 fill the GPU: eight checks per lane, in one chain
+    and in two, and the staged pass; random LLRs and syndromes."""
+    code = q.create_code_from(synth.rate002_code(2049))
+    F, g = 24, torch.Generator(device="cuda")
+    g.manual_seed(5)
+    llr = torch.randn(F * code.n, generator=g, device="cuda") * 0.5
+    syn = torch.randint(-2 ** 31, 2 ** 31, (F * ((code.m + 31) // 32),), generator=g, device="cuda",
+                        dtype=torch.int64).to(torch.int32)
+    out = []
+    for groups, cn in ((1, 0), (2, 0), (1, 160), (1, 256)):
+        dec = q.Decoder(code, F, q.qcldpc_params_init(msg_format=fmt, frame_groups=groups, cn_threads=cn))
+        dec.decode(llr, syn, 15)
+        torch.cuda.synchronize()
+        out.append((dec.keys.cpu(), dec.converged.cpu(), dec.iters.cpu()))
+    for o in out[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(o, out[0]))
 
 
 @pytest.mark.parametrize("maker, Z, groups", [

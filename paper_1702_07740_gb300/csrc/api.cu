@@ -129,7 +129,12 @@ int upload_tables(qcldpc_code *code) {
     put(H.d1_shift, &T.d1_shift);
     put(H.d1_row, &T.d1_row);
     put(H.d1_col, &T.d1_col);
+    // A copy from pageable memory may return while its last part is still on
+    // the way to the device, and a non-blocking stream does not wait for the
+    // legacy stream that carries it: the first launch there could read the
+    // tables of the block's previous owner. So the copy ends before any launch.
     err = cudaMemcpy(base + off, stage.data(), total, cudaMemcpyHostToDevice);
+    if (err == cudaSuccess) err = cudaStreamSynchronize(cudaStreamLegacy);
     if (err != cudaSuccess) {
         arena_give(off);
         std::memset(&T.row_ptr, 0, sizeof(T) - offsetof(Table, row_ptr));

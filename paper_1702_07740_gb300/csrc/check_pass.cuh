@@ -377,13 +377,13 @@ __device__ __forceinline__ bool cn_compute(const Table &T, const Work &W, int f,
                         const M ea = Codec<M>::enc(__uint_as_float(fbits(mag.x) ^ ska), W);
                         const M eb = Codec<M>::enc(__uint_as_float(fbits(mag.y) ^ skb), W);
                         if constexpr (FUSE) {
-                            float da = Codec<M>::dec(ea, W), db = Codec<M>::dec(eb, W);
+                            float da = msg_first(ea, W), db = msg_first(eb, W);
                             if constexpr (kReadMsg) {
                                 da = msg_change(ea, pM[k][c * nt], W);
                                 db = msg_change(eb, pM[k][(c + 1) * nt], W);
                             }
-                            const float la = pL[k][c * nt] + da + 0.0f;  // -0 -> +0
-                            const float lb = pL[k][(c + 1) * nt] + db + 0.0f;
+                            const float la = post_add(pL[k][c * nt], da);
+                            const float lb = post_add(pL[k][(c + 1) * nt], db);
                             float *const pa2 = Lb + (oa[k] + c * nt), *const pb2 = pa2 + nt;
                             // position shift + i of the doubled row; its twin lies Z away
                             const int qa = sh[k] + ia, qb = sh[k] + ib;

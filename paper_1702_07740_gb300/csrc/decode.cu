@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(kThreads) lvn_kernel(const __grid_constant__ T
         for (int u = 0; u < kVnVpt; u++) {
             int idx = j0 + u * kThreads - e.shift;
             if (idx < 0) idx += Z;
-            d[u] += Codec<M>::dec(nk[idx], W) - (t > 1 ? Codec<M>::dec(ok[idx], W) : 0.0f);
+            d[u] += t > 1 ? msg_change(nk[idx], ok[idx], W) : msg_first(nk[idx], W);
         }
     }
     if (!touched) return;
@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(kThreads) lvn_kernel(const __grid_constant__ T
     for (int u = 0; u < kVnVpt; u++) {
         const int j = j0 + u * kThreads;
         if (j < Z) {
-            const float lvj = L[j] + d[u] + 0.0f;  // -0 -> +0
+            const float lvj = post_add(L[j], d[u]);
             L[j] = lvj;
             L[j + Z] = lvj;
         }

@@ -363,7 +363,14 @@ struct Codec<int8_t> {
     }
 };
 
-// Stored message `now` less stored message `old`, as lvn_kernel subtracts them.
+// What a stored message adds to its node's posterior in layered decoding:
+// itself at iteration 1, and its change from the stored message `old` later.
+// Every rounding is written out (an int8 code times its quantum could otherwise
+// be contracted with whatever adds it), so that lvn_kernel and the check pass
+// that updates the posteriors itself (cn_group_kernel) give the same bits.
+__device__ __forceinline__ float msg_first(float now, const Work &) { return now; }
+__device__ __forceinline__ float msg_first(__half now, const Work &) { return __half2float(now); }
+__device__ __forceinline__ float msg_first(int8_t now, const Work &W) { return __fmul_rn((float)now, W.qstep); }
 __device__ __forceinline__ float msg_change(float now, float old, const Work &) { return now - old; }
 __device__ __forceinline__ float msg_change(__half now, __half old, const Work &) {
     return __half2float(now) - __half2float(old);
@@ -371,6 +378,9 @@ __device__ __forceinline__ float msg_change(__half now, __half old, const Work &
 __device__ __forceinline__ float msg_change(int8_t now, int8_t old, const Work &W) {
     return __fmaf_rn((float)now, W.qstep, -__fmul_rn((float)old, W.qstep));
 }
+// Posterior lv plus the (summed) change d of its messages; -0 -> +0, so that
+// sgn(0) = +1 everywhere.
+__device__ __forceinline__ float post_add(float lv, float d) { return __fadd_rn(__fadd_rn(lv, d), 0.0f); }
 
 // The integer a stored message adds to its node's accumulator: the stored
 // value in units of acc_inv (the int8 code itself; FP32 and FP16 values

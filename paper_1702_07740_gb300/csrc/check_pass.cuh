@@ -288,6 +288,17 @@ __device__ __forceinline__ bool cn_compute(const Table &T, const Work &W, int f,
 #pragma unroll
         for (int k = 0; k < NH; k++) sh[k] = oa[k] % (2 * Z);
     }
+    // FUSE: the change of heavy message k of the thread's check c (check i of
+    // the row, its new message e) goes into both copies of its node's posterior
+    [[maybe_unused]] auto add_change = [&](int k, int c, int i, M e, bool valid) {
+        float d;
+        if constexpr (kReadMsg) d = msg_change(e, pM[k][c * nt], W);
+        else d = msg_first(e, W);
+        const float l = post_add(pL[k][c * nt], d);
+        float *const p = Lb + (oa[k] + c * nt);
+        // position shift + i of the doubled row; its twin lies Z away
+        if (valid) p[0] = l, p[sh[k] + i < Z ? Z : -Z] = l;
+    };
     // syndrome words of the owned checks (check c of this thread sits c * ws
     // words after the first), loaded while the copies are in flight; rows
     // with a degree-1 node have the bit folded into its sign (syn_folded)
@@ -377,18 +388,8 @@ __device__ __forceinline__ bool cn_compute(const Table &T, const Work &W, int f,
                         const M ea = Codec<M>::enc(__uint_as_float(fbits(mag.x) ^ ska), W);
                         const M eb = Codec<M>::enc(__uint_as_float(fbits(mag.y) ^ skb), W);
                         if constexpr (FUSE) {
-                            float da = msg_first(ea, W), db = msg_first(eb, W);
-                            if constexpr (kReadMsg) {
-                                da = msg_change(ea, pM[k][c * nt], W);
-                                db = msg_change(eb, pM[k][(c + 1) * nt], W);
-                            }
-                            const float la = post_add(pL[k][c * nt], da);
-                            const float lb = post_add(pL[k][(c + 1) * nt], db);
-                            float *const pa2 = Lb + (oa[k] + c * nt), *const pb2 = pa2 + nt;
-                            // position shift + i of the doubled row; its twin lies Z away
-                            const int qa = sh[k] + ia, qb = sh[k] + ib;
-                            if (va) pa2[0] = la, pa2[qa < Z ? Z : -Z] = la;
-                            if (vb) pb2[0] = lb, pb2[qb < Z ? Z : -Z] = lb;
+                            add_change(k, c, ia, ea, va);
+                            add_change(k, c + 1, ib, eb, vb);
                         }
                         st_if(oM[k] + c * nt, ea, va);
                         st_if(oM[k] + (c + 1) * nt, eb, vb);
@@ -459,6 +460,7 @@ __device__ __forceinline__ bool cn_compute(const Table &T, const Work &W, int f,
                     if (k < NH) {
                         const float mag = psi_f(fmaxf(s1, W.xmin_h));
                         const M e = Codec<M>::enc(__uint_as_float(fbits(mag) ^ sk), W);
+                        if constexpr (FUSE) add_change(k, c, i, e, valid);
                         if (valid) {
                             oM[k][c * nt] = e;
                             if (accum) red_add(accb + (oa[k] + c * nt), acc_value(e, W));

@@ -1,5 +1,9 @@
 """Layered decoding: row groups whose check pass updates the posteriors itself
 give the bits of the check pass followed by the posterior pass."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -9,6 +13,7 @@ from bench import layered_launches
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
+from paper_1702_07740_gb300 import build  # noqa: E402
 from paper_1702_07740_gb300 import qcldpc as q  # noqa: E402
 from test_gpu_kernel_edges import odd_code  # noqa: E402
 
@@ -64,3 +69,15 @@ def test_fused_groups_have_the_bits_of_the_separate_update(maker, Z, fmt, step):
         np.testing.assert_array_equal(post.view(np.int32), ref[:, :n].copy().view(np.int32))
         hard, _ = decode(d, llr[:, :n].copy(), own, iters, False, msg_format=fmt, msg_step=step)
         np.testing.assert_array_equal(hard, keys)
+
+
+def test_checks_evaluated_one_at_a_time_update_the_posteriors_too(tmp_path):
+    """A build without packed pairs (an option of tuning builds) takes the
+    scalar form of the check pass; its fused groups match the oracle."""
+    lib = build.build(extra_flags=["-DQCLDPC_CN_PAIR=0"], out_dir=str(tmp_path))
+    tests = os.path.dirname(os.path.abspath(__file__))
+    r = subprocess.run([sys.executable, "-m", "pytest", "-q", "-m", "gpu", "-p", "no:cacheprovider",
+                        os.path.join(tests, "test_gpu_kernel_edges.py"), os.path.abspath(__file__),
+                        "-k", "one_row_groups or separate_update"],
+                       env=dict(os.environ, QCLDPC_LIB=lib), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-2000:]

@@ -211,7 +211,10 @@ __global__ void __launch_bounds__(qc::kCnDirectThreads, kCdMinBlocks)
     // warp has a failed check, and a store from each queued up in the L2 at
     // the one word (n = 10^6, 16 frames: 185 us a pass against 105 us).
     __shared__ int s_failed;
-    if (!W.side) pdl_launch_dependents();  // see cn_tma_kernel
+    // The posterior pass may be scheduled once the last block runs, unless other
+    // chains run beside this one: its waiting blocks would keep theirs off the
+    // SMs (see cn_tma_kernel, whose blocks are larger and gain nothing by it).
+    if (!W.side) pdl_launch_dependents();
     if (threadIdx.x == 0) s_failed = 0;
     __syncthreads();
     pdl_wait();  // after a programmatic edge: the previous posterior pass is complete

@@ -589,12 +589,13 @@ template <int MAXD, typename M, int NT, bool SOFT>
 __global__ void __launch_bounds__(kCnThreads, NT ? QCLDPC_CN_TMA_MINBLOCKS : QCLDPC_CN_FIT_MINBLOCKS)
     cn_tma_kernel(const __grid_constant__ Table T, const __grid_constant__ Work W) {
     extern __shared__ __align__(128) unsigned char smem[];
-    // The next step may be scheduled as soon as the last block runs; it waits
-    // for this pass. Not beside other chains: its waiting blocks would keep
-    // theirs off the SMs (multi-edge code, two groups of 8 frames, 65
-    // iterations: 10.6 ms, and 8.2 ms with a control kernel in between), so
-    // there it is scheduled when this pass ends.
-    if (!W.side) pdl_launch_dependents();
+    // The next step is scheduled as this pass's blocks end. Triggered at the
+    // start instead, its blocks would wait in slots that this pass's blocks, and
+    // those of decodes on other streams, could run in: soft decodes of one
+    // multi-edge frame each, 60 iterations, took 3.29 ms on 4 streams and 6.91 on
+    // 8 that way, and 2.92 and 6.17 this way; alone 1.79 and 1.80. Thirty
+    // iterations of 26 such frames with Z = 9 took 1.84 and 1.63 ms in one
+    // decode, of 38 frames of 19 rows with Z = 559 0.37 and 0.39.
     pdl_wait();  // after a programmatic edge: the previous variable pass is complete
     const int f = blockIdx.z;
     const bool running = W.active[f] != 0;
@@ -647,7 +648,6 @@ template <typename M, bool SOFT>
 __global__ void __launch_bounds__(kCnThreads, QCLDPC_CN_FIT_MINBLOCKS)
     cn_group_kernel(const __grid_constant__ Table T, const __grid_constant__ Work W) {
     extern __shared__ __align__(128) unsigned char smem[];
-    if (!W.side) pdl_launch_dependents();  // see cn_tma_kernel
     pdl_wait();  // the previous group's posteriors are complete and visible
     const int f = blockIdx.z;
     if (W.active[f] == 0) return;  // block-uniform

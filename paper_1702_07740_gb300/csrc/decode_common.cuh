@@ -176,7 +176,7 @@ struct Work {
     int32_t *acc;          // [F][n_hcols][2Z]
     float acc_scale;       // FP32 / FP16 messages: fixed-point scale 2^k (int8: unused)
     float acc_inv;         // 2^-k, or the int8 quantum (the sum then counts quanta)
-    int32_t side;          // 1: other chains run beside this one (see cn_tma_kernel)
+    int32_t side;          // 1: other chains run beside this one (see cn_direct_kernel)
     int32_t accum;         // 1: accumulated posteriors; 0: separate summing variable pass
     // Bounded waits of the staged check pass: polls before giving up, and a
     // test switch (QCLDPC_TEST_STALL=1 in the environment) under which each

@@ -93,7 +93,7 @@ int upload_tables(qcldpc_code *code) {
                          bytes_of(H.col_ptr) + bytes_of(H.hcol_base) + bytes_of(H.col_kind) +
                          bytes_of(H.rows) + bytes_of(H.row_off_a) + bytes_of(H.row_off_b) +
                          bytes_of(H.cols) + bytes_of(H.col_row) + bytes_of(H.d1_shift) +
-                         bytes_of(H.d1_row) + bytes_of(H.d1_col);
+                         bytes_of(H.d1_syn) + bytes_of(H.d1_col);
     size_t off;
     if (!arena_take(total, &off))
         return fail(QCLDPC_E_NOMEM, "code tables: the device table arena (64 MiB) is full");
@@ -127,7 +127,7 @@ int upload_tables(qcldpc_code *code) {
     put(H.cols, &T.cols);
     put(H.col_row, &T.col_row);
     put(H.d1_shift, &T.d1_shift);
-    put(H.d1_row, &T.d1_row);
+    put(H.d1_syn, &T.d1_syn);
     put(H.d1_col, &T.d1_col);
     // A copy from pageable memory may return while its last part is still on
     // the way to the device, and a non-blocking stream does not wait for the
@@ -253,7 +253,6 @@ extern "C" int qcldpc_create_code(int mb, int nb, int Z, int n_circ,
         if (col_count[circ_col[h]] == 1) {
             did[h] = n_d1;
             H.d1_shift.push_back(circ_shift[h]);
-            H.d1_row.push_back(circ_row[h]);
             H.d1_col.push_back(circ_col[h]);
             H.col_kind[circ_col[h]] = -n_d1 - 2;
             n_d1++;
@@ -293,6 +292,11 @@ extern "C" int qcldpc_create_code(int mb, int nb, int Z, int n_circ,
         }
         H.row_ptr[mb] = (int32_t)H.rows.size();
         T.max_row_deg = max_deg;
+        H.d1_syn.assign(n_d1, -1);
+        for (int r = 0; r < mb; r++) {
+            const int d1 = H.row_ptr[r] + H.row_nh[r], nd = H.row_ptr[r + 1] - d1;
+            if (syn_folded(nd)) H.d1_syn[H.rows[d1].id] = r * Z;
+        }
     }
     // Check-node blocks visit rows in this order: rows of one shape (heavy
     // and degree-1 counts) are adjacent, so blocks resident together tend to

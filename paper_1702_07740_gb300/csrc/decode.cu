@@ -109,18 +109,17 @@ __global__ void __launch_bounds__(kThreads) init_kernel(const __grid_constant__ 
         const int64_t f = q / ((int64_t)T.n_d1 * W.ZW);
         const int64_t rem = q - f * T.n_d1 * W.ZW;
         const int k = (int)(rem / W.ZW), wd = (int)(rem - (int64_t)k * W.ZW);
-        const int i = wd * 32 + lane;
+        const int i = wd * 32 + lane, sc = T.d1_syn[k];
         bool neg = false;
         if (i < Z) {
             int vo = i + T.d1_shift[k];
             if (vo >= Z) vo -= Z;
+            const bool syn = sc >= 0 && syn_sign(W, f, sc + i) != 0;
             const float qv = W.llr[f * W.n + (int64_t)T.d1_col[k] * Z + vo];
             const float a = fmaxf(fminf(fabsf(qv) * kLog2e, W.clip), W.xmin);
             const float p = psi_f(a);
             const size_t off = ((size_t)f * T.n_d1 + k) * Z + i;
-            neg = qv < 0.0f;
-            const int r = T.d1_row[k];
-            if (row_syn_folded(T, r)) neg ^= syn_sign(W, f, r * Z + i) != 0;
+            neg = (qv < 0.0f) != syn;
             W.phiq[off] = neg ? -p : p;
             if (W.soft) W.post1[off] = qv;  // iteration-0 posterior, buffer 0
         }
@@ -490,8 +489,8 @@ __global__ void __launch_bounds__(kThreads) final_kernel(const __grid_constant__
                 const uint32_t word =
                     W.bits[(((size_t)b * W.n_frames + f) * T.n_d1 + d) * W.ZW + (i >> 5)];
                 dec = (word >> (i & 31)) & 1u;
-                const int r = T.d1_row[d];
-                if (row_syn_folded(T, r)) dec ^= syn_sign(W, f, r * Z + i) != 0;
+                const int sc = T.d1_syn[d];
+                if (sc >= 0) dec ^= syn_sign(W, f, sc + i) != 0;
             }
         }
         const uint32_t word = __ballot_sync(0xffffffffu, dec);
@@ -1757,17 +1756,17 @@ __global__ void __launch_bounds__(kThreads) pool_load_kernel(const __grid_consta
         const int64_t rem = qw - q * T.n_d1 * W.ZW;
         const int k = (int)(rem / W.ZW), wd = (int)(rem - (int64_t)k * W.ZW);
         const int64_t f = slots[q];
-        const int i = wd * 32 + lane;
+        const int i = wd * 32 + lane, sc = T.d1_syn[k];
         bool neg = false;
         if (i < Z) {
             int vo = i + T.d1_shift[k];
             if (vo >= Z) vo -= Z;
+            const int c = sc + i;
+            const bool syn = sc >= 0 && (syn_src[q * W.words_m + (c >> 5)] >> (c & 31)) & 1u;
             const float qv = llr_src[q * N + (int64_t)T.d1_col[k] * Z + vo];
             const float a = fmaxf(fminf(fabsf(qv) * kLog2e, W.clip), W.xmin);
             const float p = psi_f(a);
-            neg = qv < 0.0f;
-            const int r = T.d1_row[k], c = r * Z + i;
-            if (row_syn_folded(T, r)) neg ^= (syn_src[q * W.words_m + (c >> 5)] >> (c & 31)) & 1u;
+            neg = (qv < 0.0f) != syn;
             W.phiq[((size_t)f * T.n_d1 + k) * Z + i] = neg ? -p : p;
         }
         const uint32_t word = __ballot_sync(0xffffffffu, neg);
@@ -1814,8 +1813,8 @@ __global__ void __launch_bounds__(kThreads) pool_collect_kernel(
                 const uint32_t word =
                     W.bits[(((size_t)b * W.n_frames + f) * T.n_d1 + d) * W.ZW + (i >> 5)];
                 dec = (word >> (i & 31)) & 1u;
-                const int r = T.d1_row[d];
-                if (row_syn_folded(T, r)) dec ^= syn_sign(W, f, r * Z + i) != 0;
+                const int sc = T.d1_syn[d];
+                if (sc >= 0) dec ^= syn_sign(W, f, sc + i) != 0;
             }
         }
         const uint32_t word = __ballot_sync(0xffffffffu, dec);

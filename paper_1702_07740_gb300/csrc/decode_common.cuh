@@ -15,6 +15,7 @@ namespace {
 
 using qc::Table;
 using qc::exact_shape;
+using qc::syn_folded;
 
 // Launch shapes (overridable at build time for tuning sweeps). Defaults
 // from a sweep at Z = 20,000 with 16 frames on GB300.
@@ -324,19 +325,6 @@ __device__ __forceinline__ uint32_t fbits(float x) { return __float_as_uint(x); 
 // Syndrome bit of check c (row * Z + offset) of frame f, as a sign bit.
 __device__ __forceinline__ uint32_t syn_sign(const Work &W, int64_t f, int c) {
     return __ldg(W.syn + f * W.words_m + (c >> 5)) << (31 - (c & 31)) & kSign;
-}
-
-// A check with one degree-1 neighbour p keeps its syndrome bit folded into
-// that neighbour: phiq holds psi(|Q_p|) with the sign of Q_p times the
-// syndrome sign, and `bits` the decision C_p plus (mod 2) the syndrome bit.
-// The sign total of the check, its parity and the choice between sgn(m_cp)
-// and sgn(Q_p) then come out without the check pass ever reading the
-// syndrome (one unaligned load, a range test and a shift per check less);
-// outputs of degree-1 nodes take the bit out again. nd: the row's degree-1
-// circulants.
-__host__ __device__ constexpr bool syn_folded(int nd) { return nd == 1; }
-__device__ __forceinline__ bool row_syn_folded(const Table &T, int r) {
-    return syn_folded(T.row_ptr[r + 1] - T.row_ptr[r] - T.row_nh[r]);
 }
 
 // Storage formats of the check-to-variable messages (computation is FP32):

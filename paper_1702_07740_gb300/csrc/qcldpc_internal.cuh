@@ -55,6 +55,16 @@ __host__ __device__ constexpr bool exact_shape(int nh, int nd) {
     return (nd == 1 && nh >= 1 && nh <= 4) || (nd == 0 && nh >= 2 && nh <= 4);
 }
 
+// A check with one degree-1 neighbour p keeps its syndrome bit folded into
+// that neighbour: phiq holds psi(|Q_p|) with the sign of Q_p times the
+// syndrome sign, and `bits` the decision C_p plus (mod 2) the syndrome bit.
+// The sign total of the check, its parity and the choice between sgn(m_cp)
+// and sgn(Q_p) then come out without the check pass ever reading the
+// syndrome (one unaligned load, a range test and a shift per check less);
+// outputs of degree-1 nodes take the bit out again. nd: the row's degree-1
+// circulants.
+__host__ __device__ constexpr bool syn_folded(int nd) { return nd == 1; }
+
 // Code tables as the kernels see them: scalars, and pointers into the code's
 // block of the library's static device table arena (uploaded on the first
 // call that launches work). Passed to kernels by value as a
@@ -89,7 +99,8 @@ struct Table {
     const ColEnt *cols;        // [n_h] heavy circulants by heavy column
     const int32_t *col_row;    // [n_h] base row of each cols[] entry
     const int32_t *d1_shift;   // [n_d1]
-    const int32_t *d1_row;     // [n_d1]
+    const int32_t *d1_syn;     // [n_d1] first check of the circulant's row if its node carries the
+                               // check's syndrome bit (syn_folded), else -1
     const int32_t *d1_col;     // [n_d1]
 };
 
@@ -108,7 +119,7 @@ struct HostTable {
     std::vector<RowEnt> rows;
     std::vector<int32_t> row_off_a, row_off_b;
     std::vector<ColEnt> cols;
-    std::vector<int32_t> col_row, d1_shift, d1_row, d1_col;
+    std::vector<int32_t> col_row, d1_shift, d1_syn, d1_col;
 };
 
 // Uploads the code's tables to the device table arena if they are not there

@@ -1,7 +1,7 @@
 // Syndrome and 8-dimensional reconciliation kernels.
 //
 // * qcldpc_syndrome: s = H x over GF(2) for the QC expansion of Sec. III-C,
-//   one thread per check node, results packed with a warp ballot.
+//   one thread per word of 32 check nodes or, where rows are short, per check.
 // * qcldpc_bob_message_8d / qcldpc_llr_8d: Sec. II-C. Bob sends M = U Y with
 //   U_j = (-1)^{C_j}; Alice divides, R = M X^{-1} = M conj(X) / |X|^2, and
 //   with sigma_N^2 = 8 sigma_Z^2 / |X|^2 the channel LLR of Step 1 of
@@ -98,6 +98,50 @@ __global__ void __launch_bounds__(128) syndrome_kernel(const __grid_constant__ q
         r++;
     }
     syn[(int64_t)blockIdx.y * words_m + w] = out;
+}
+
+// One thread per check, results packed with a warp ballot: for rows so short
+// that a word of the other form would walk many of them one after the other.
+__global__ void __launch_bounds__(256) syndrome_bit_kernel(const __grid_constant__ qc::Table T,
+                                                           const uint32_t *__restrict__ bits,
+                                                           uint32_t *__restrict__ syn,
+                                                           int64_t words_n, int64_t words_m) {
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int Z = T.Z;
+    const bool on = c < (int64_t)T.mb * Z;
+    const uint32_t *fb = bits + (int64_t)blockIdx.y * words_n;
+    uint32_t par = 0;
+    if (on) {
+        const int r = (int)(c / Z), i = (int)(c - (int64_t)r * Z);
+        const int ke = T.row_ptr[r + 1];
+        for (int k = T.row_ptr[r]; k < ke; k++) {
+            const qc::RowEnt e = T.rows[k];
+            int j = i + e.shift;
+            if (j >= Z) j -= Z;
+            const int64_t v = (int64_t)e.col * Z + j;
+            par ^= __ldg(fb + (v >> 5)) >> (v & 31) & 1u;
+        }
+    }
+    const uint32_t word = __ballot_sync(0xffffffffu, par);
+    if ((threadIdx.x & 31) == 0 && on) syn[(int64_t)blockIdx.y * words_m + (c >> 5)] = word;
+}
+
+// Whether a syndrome call takes the word form. A word meets `seg` rows at most
+// (it starts at a multiple of gcd(Z, 32) in a row) and its thread reads their
+// circulants one after the other, so the word form's latency grows with their
+// product. A few thousand checks of 7 circulants took it 53 us at Z = 1, 10.3 at
+// 8 and 15 (28 reads), 6.2 at 16 (14), and the bit form 4.8 (the call's host
+// time) at each of them. Up to 18 reads the word form is at most 1.5 us behind
+// there and ahead from a few hundred thousand checks on (one multi-edge frame,
+// Z = 625, 16 reads: 6.2 and 10.3 us). Above a million checks the number of
+// reads counts, and the word form is ahead from Z = 6 on (Z = 8, 7 circulants,
+// 6.4 million checks: 37 and 62 us), not below (Z = 4, 3 circulants, 3.2
+// million: 28.7 and 20.6).
+bool syndrome_by_words(const qc::Table &T, int n_frames) {
+    int g = 1;
+    while (g < 32 && T.Z % (2 * g) == 0) g *= 2;
+    const int seg = 1 + (32 - g + T.Z - 1) / T.Z;
+    return seg * T.max_row_deg <= 18 || (seg <= 6 && (int64_t)n_frames * T.mb * T.Z >= 1 << 20);
 }
 
 __global__ void __launch_bounds__(256) bob8_kernel(const float4 *__restrict__ y,
@@ -289,9 +333,12 @@ extern "C" int qcldpc_syndrome(const qcldpc_code *code, const uint32_t *bits_dev
     if (n_frames == 0) return QCLDPC_OK;
     if (int st = upload_tables(const_cast<qcldpc_code *>(code))) return st;
     const int64_t words_n = (code->n + 31) / 32, words_m = (code->m + 31) / 32;
-    dim3 grid((unsigned)((words_m + 127) / 128), (unsigned)n_frames);
-    syndrome_kernel<<<grid, 128, 0, (cudaStream_t)stream>>>(code->tab, bits_dev, syn_dev,
-                                                           words_n, words_m);
+    const bool words = syndrome_by_words(code->tab, n_frames);
+    const int nt = words ? 128 : 256;
+    const int64_t threads = words ? words_m : code->m;
+    dim3 grid((unsigned)((threads + nt - 1) / nt), (unsigned)n_frames);
+    auto kernel = words ? syndrome_kernel : syndrome_bit_kernel;
+    kernel<<<grid, nt, 0, (cudaStream_t)stream>>>(code->tab, bits_dev, syn_dev, words_n, words_m);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return cuda_fail(err, "syndrome: launch");
     return QCLDPC_OK;

@@ -193,21 +193,31 @@ class ClockSampler:
 
 # ------------------------------------------------------- algorithmic bytes
 
-def pass_bytes(Z: int, n_h: int, n_d1: int, n_hcols: int, mb: int, msg_bytes: int = 4,
+def syndrome_rows(d) -> int:
+    """Base rows whose checks read the syndrome in every pass: those without
+    exactly one degree-1 circulant (the others' bits are folded into the sign of
+    their degree-1 node's Phi value)."""
+    row, col = np.asarray(d["row"]), np.asarray(d["col"])
+    single = np.bincount(col, minlength=d["nb"])[col] == 1
+    return int((np.bincount(row[single], minlength=d["mb"]) != 1).sum())
+
+
+def pass_bytes(Z: int, n_h: int, n_d1: int, n_hcols: int, syn_rows: int, msg_bytes: int = 4,
                accumulate: bool = True):
     """Bytes one frame's check-node / variable-node pass must move.
 
     Check pass: read and write every heavy message (n_h Z messages each way),
     read the degree-1 Phi values (n_d1 Z floats), the heavy posteriors once
-    (n_hcols Z floats), the syndrome (mb Z bits) and previous degree-1
-    decisions (n_d1 Z bits), write new decisions (n_d1 Z bits).
+    (n_hcols Z floats), the syndrome of the rows that need it (syn_rows Z
+    bits) and previous degree-1 decisions (n_d1 Z bits), write new decisions
+    (n_d1 Z bits).
     Variable pass, separate: read every heavy message once, the heavy channel
     LLRs, and write the heavy posteriors (stored twice, 2 x 4 bytes).
     Variable pass, accumulated: read the two integer partial sums of every
     heavy node and clear them (16 bytes), read its channel LLR and write its
     posterior twice.
     """
-    cn = 2 * msg_bytes * n_h * Z + 4 * (n_d1 * Z + n_hcols * Z) + (mb * Z + 2 * n_d1 * Z) / 8
+    cn = 2 * msg_bytes * n_h * Z + 4 * (n_d1 * Z + n_hcols * Z) + (syn_rows * Z + 2 * n_d1 * Z) / 8
     if accumulate:
         vn = (16 + 4 + 8) * n_hcols * Z
     else:
@@ -215,13 +225,13 @@ def pass_bytes(Z: int, n_h: int, n_d1: int, n_hcols: int, mb: int, msg_bytes: in
     return cn, vn
 
 
-def iteration_bytes(Z: int, n_h: int, n_d1: int, n_hcols: int, mb: int, msg_bytes: int = 4):
+def iteration_bytes(Z: int, n_h: int, n_d1: int, n_hcols: int, syn_rows: int, msg_bytes: int = 4):
     """Algorithmic bytes of one flooding iteration of one frame: every heavy
     message read and written once, the degree-1 Phi values read, the heavy
-    posteriors read and written with their channel LLRs, the syndrome and the
-    degree-1 decisions in and out."""
+    posteriors read and written with their channel LLRs, the syndrome of the
+    rows that need it and the degree-1 decisions in and out."""
     return (2 * msg_bytes * n_h * Z + 4 * n_d1 * Z + 12 * n_hcols * Z
-            + (mb * Z + 2 * n_d1 * Z) / 8)
+            + (syn_rows * Z + 2 * n_d1 * Z) / 8)
 
 
 def launch_count(group_passes, per_pass: int, unroll: int) -> int:
@@ -249,6 +259,15 @@ def layered_launches(d, groups: int) -> int:
         fuses = exact[rows].all() and len(np.unique(cols)) == len(cols)
         total += 1 if fuses else 2
     return total
+
+
+def kernels_per_pass(args, d) -> int:
+    """Kernels of one loop pass of a chain. Flooding: check pass and posterior
+    pass, which takes the loop's decisions (with a separate variable pass a
+    control step too); layered: see layered_launches."""
+    if args.schedule == "layered":
+        return layered_launches(d, args.layers or d["mb"])
+    return 2 if args.vn_pass == "accumulate" else 3
 
 
 def groups_of(args, F):
@@ -501,12 +520,8 @@ def run_ours(args, world, rank, local):
         group_passes[b] = [int(its[firsts[g]:firsts[g + 1]].max()) + 1 for g in range(G)]
     frames_total = len(used) * F
     fer = frame_err / frames_total
-    # per step: llr, and per frame group init + final; per loop pass of a
-    # group's own loop, check pass + posterior pass (flooding; with a separate
-    # variable pass a control step too) or test pass + control + 1 or 2 per row
-    # group (layered)
-    per_pass = (layered_launches(d, args.layers or d["mb"]) if layered
-                else 2 if args.vn_pass == "accumulate" else 3)
+    # per step: llr, per frame group init + final, and its loop passes' kernels
+    per_pass = kernels_per_pass(args, d)
     # each group's loop runs flooding iterations four per trip until its own
     # frames have stopped, and the stream launch mode enqueues max_iter + 1
     # passes; passes after every frame stopped exit at once but still launch
@@ -583,7 +598,7 @@ def run_ours(args, world, rank, local):
     col_count = np.bincount(d["col"], minlength=d["nb"])
     heavy = col_count != 1
     shape = dict(Z=d["Z"], n_h=int(heavy[d["col"]].sum()), n_d1=int((~heavy[d["col"]]).sum()),
-                 n_hcols=int(heavy.sum()), mb=d["mb"],
+                 n_hcols=int(heavy.sum()), syn_rows=syndrome_rows(d),
                  msg_bytes={"fp32": 4, "fp16": 2, "int8": 1}[args.msg_format])
     cn_b, vn_b = pass_bytes(**shape, accumulate=args.vn_pass == "accumulate" and not layered)
     it_b = iteration_bytes(**shape)

@@ -188,7 +188,14 @@ typedef struct qcldpc_params {
        changes a result bit (qcldpc_autotune_shapes picks them by time). */
     int32_t cn_threads;  /* threads per check-pass block: a multiple of 32,
                             32..256; a block evaluates 2 to 8 checks per thread
-                            of one base row */
+                            of one base row. It also picks the kernel: where
+                            flooding has a check pass that loads its operands
+                            straight into registers (every base row with at most
+                            four heavy and one degree-1 circulants), 0 and widths
+                            up to 128 take it and larger ones take the pass that
+                            stages them in shared memory (99.8 us an iteration
+                            of 16 frames of n = 10^6 instead of 86.9); layered
+                            decoding always stages */
     int32_t vn_nodes;    /* variable pass: heavy nodes per thread, 1..3 */
     int32_t vn_split;    /* variable pass: 1 = a thread adds both partial sums
                             of its nodes, 2 = two thread groups, one per
@@ -436,15 +443,16 @@ int qcldpc_time_passes(const qcldpc_code *code, int n_frames, void *workspace_de
  * expose it, or a process whose device memory is reserved once at start-up
  * and may not grow. This entry point computes exactly what qcldpc_decode
  * computes (same kernels, passes enqueued one by one on `stream`, no graph
- * objects), but keeps its scratch in a static 16 MiB device array inside the
- * library instead of a caller workspace. Every GPU that loads the library
+ * objects), but keeps its scratch in a static device array of 16.5 MiB inside
+ * the library instead of a caller workspace. Every GPU that loads the library
  * holds that array until the process exits. The caller still passes the
  * inputs and outputs described at qcldpc_decode; the array is never exposed.
  *
- * Limit: the code's workspace for n_frames (qcldpc_decode_workspace with
- * default options) must fit in 16 MiB, e.g. one frame of the rate-0.02,
- * n = 10^6 code; larger requests return QCLDPC_E_UNSUPPORTED and a message
- * naming both sizes. p->soft_output and p->launch_mode are ignored.
+ * Limit: the workspace of the n_frames as one chain with the call's message
+ * format and schedule, less the frames' control words (which the array's last
+ * 0.5 MiB hold), must fit in 16 MiB, e.g. one frame of the rate-0.02, n = 10^6
+ * code in FP32, two in int8; larger requests return QCLDPC_E_UNSUPPORTED and a
+ * message naming both sizes. p->soft_output and p->launch_mode are ignored.
  *
  * The first call on each device looks up the array's device address (with
  * that device current); make that first call before any stream capture.

@@ -6,13 +6,15 @@
 // contiguous 128-byte run. Pairs of a lane's checks are evaluated in packed
 // FP32x2 arithmetic, bit for bit as in the staged pass (check_pass.cuh), and
 // the next pair's operands are loaded before a pair computes. Warps share
-// nothing but one flag, so there is no block barrier behind a serial copy
-// set-up and no shared-memory round trip. Bounded by the latency of its loads
+// nothing but one flag, so no warp waits at a barrier for a serial copy set-up,
+// and there is no shared-memory round trip. Bounded by the latency of its loads
 // and by instruction issue: 16 frames of n = 10^6, FP32, took 102.7 us a pass
 // staged and take 89.5 us, FP16 90.9 and 83.7 (replayed alone). Without the
 // loads ahead 8 checks per lane took 103 us, and 256-thread blocks 100.6.
-// Registers: 72 (7 blocks of 128 threads); 64 spill and 80 leave too few warps
-// (5 frames 30.7, 26.7 and 26.2 us, 16 frames 85.8, 86.9 and 93.1 us an iteration).
+// Registers: 72 (7 blocks of 128 threads), where the FP32 form with 8 checks per
+// lane spills 148 bytes a thread. 64 spill 748; 80, the first without a spill,
+// leave too few warps: 85.8, 86.9 and 93.1 us an iteration of 16 frames at 64, 72
+// and 80, and 30.7, 26.7 and 26.2 of 5 frames.
 #pragma once
 
 #include "decode_common.cuh"

@@ -21,8 +21,9 @@
 //
 // One iteration t is two streaming kernels:
 //   check pass  (cn_direct_kernel or cn_tma_kernel) per check c (row r,
-//               offset i): L_vc = clip(L_v - m_cv(t-1)) for heavy neighbours v = (col, (i+s) mod Z), Phi-domain exclusive
-//               sums, m_cv(t) written back in place; decisions of the degree-1
+//               offset i): L_vc = clip(L_v - m_cv(t-1)) for heavy neighbours
+//               v = (col, (i+s) mod Z), Phi-domain exclusive sums, m_cv(t)
+//               written back in place; decisions of the degree-1
 //               neighbours of iteration t. It also evaluates the stop test of
 //               iteration t-1 (H C(t-1) = s) from the L(t-1) values it reads
 //               anyway, so the test costs no extra pass over memory.
@@ -420,8 +421,12 @@ dim3 post_grid(const Table &T, int F) {
 template <typename M>
 __global__ void __launch_bounds__(kThreads) lvn_kernel(const __grid_constant__ Table T,
                                                        const __grid_constant__ Work W) {
+    // The next group's check pass is scheduled as this pass's blocks end. Triggered
+    // at the start, its large blocks waited in the slots of other chains' check
+    // passes: 30 iterations in 7 row groups of 16 frames of n = 10^6 took 9.03 ms in
+    // two frame groups that way and 6.98 this way (7.54 in one, both ways), and of
+    // 4 frames each on 4 streams 7.54 and 5.85.
     pdl_wait();  // the group's check pass is complete and visible
-    pdl_launch_dependents();  // the next group's check pass may be scheduled; it waits for this pass
     const int f = blockIdx.z;
     if (W.active[f] == 0) return;
     const int t = W.t[f] - 1;
@@ -773,8 +778,9 @@ int cn_threads(int Z) {
 // of two. Per iteration: 16 frames of n = 10^6 99.8 us staged, 86.9 with 8;
 // one frame (3,871 warps of 8) 14.0 staged, 12.2 with 8, 13.2 with 4; 7 frames
 // of 9 rows, Z = 9,999 (1,440 a chain) 9.1 with 2, 9.9 with 4; one frame,
-// Z = 512 (98) 7.0 staged, 8.2 with 8, 5.7 with 2. Soft output, a small-batch
-// option, has the direct form for small grids only.
+// Z = 512 (98) 7.0 staged, 8.2 with 8, 5.7 with 2. Soft output has the form
+// with 2 only, which is behind on full grids: 50 iterations of 16 frames of
+// n = 10^6 took 9.50 ms staged and 10.35 with 2, of 4 frames 2.67 and 2.57.
 int cn_direct_slots(const Table &T, const Work &w, int nt_set) {
     if (w.layered || !w.accum || w.stall_extra || nt_set > qc::kCnDirectThreads || T.exact_rows != T.mb) return 0;
     const long long resident = (long long)sm_count() * (kCdMinBlocks * qc::kCnDirectThreads / 32);
@@ -902,8 +908,8 @@ cudaError_t add_loop_body(cudaGraph_t body, const qcldpc_code *code, const Work 
     // kLoopUnroll flooding iterations per trip of the WHILE body (each trip
     // costs a body relaunch, ~4 us on GB300): passes of frames that stopped
     // in an earlier iteration of the trip exit at once, and the last control
-    // step decides whether another trip runs. A layered iteration is 2 + 2G
-    // launches, so its body holds one.
+    // step decides whether another trip runs. A layered iteration is 2 launches
+    // and one or two per row group, so its body holds one.
     const int unroll = w0.layered ? 1 : kLoopUnroll;
     const std::vector<char> fuses = fused_groups(code, w0.layered ? w0.ngroups : 0);
     cudaGraphNode_t prev = nullptr;
@@ -1312,10 +1318,10 @@ extern "C" int qcldpc_decode_soft(const qcldpc_code *code, const float *llr_dev,
 // The graph holds, for every code (or every frame group of one code), the
 // chain a one-code decode runs: initialisation, a device-side loop (a
 // conditional WHILE node) over the flooding passes (check pass and posterior
-// pass, kLoopUnroll times per trip) whose control steps end it once the chain's own frames have stopped, and the output step. The
-// chains are independent branches, so the small grids of short codes fill
-// the GPU together and one chain's short steps run inside another's check
-// pass. Each frame keeps its own iteration counter and stop test, so its
+// pass, kLoopUnroll times per trip) whose stop decisions end it once the
+// chain's own frames have stopped, and the output step. The chains are
+// independent branches, so the small grids of short codes fill the GPU
+// together and one chain's short steps run inside another's check pass. Each frame keeps its own iteration counter and stop test, so its
 // result is the one a one-code decode of the same frames gives.
 namespace {
 
@@ -1514,7 +1520,7 @@ extern "C" int qcldpc_autotune(const qcldpc_code *code, const float *llr_dev,
     else qcldpc_params_init(&base);
     const int mb = code->tab.mb;
     // 0: flooding, else layered with that many row groups (at most 64: a
-    // group costs two launches per iteration)
+    // group costs one or two launches per iteration)
     const int want[4] = {0, 2, 7, std::min(mb, 64)};
     if (times_ms)
         for (int i = 0; i < 4; i++) times_ms[i] = NAN;
